@@ -52,6 +52,10 @@ struct Cap {
     static constexpr int STACK = TP <= 4 ? STACK_CAP : 4 * STACK_CAP;
 };
 constexpr int CHUNK = 4;
+// From this radius pass on (from the second one for listed cells) a search also tests nodes and points against the balls
+// of the cell's vertices: the cells that get there bound a void beside dense halos, and without it collect thousands of
+// halo points in passes of 256.
+constexpr int BALL_PASS = 2;
 
 template <typename CT> struct Prec;
 template <> struct Prec<float> {
@@ -99,7 +103,10 @@ struct WarpSmem {
         } em;
     } u;
     uint32_t bnd[K::MAXT];       // boundary records of a cut: x, y, kept neighbour slot, its edge index
-    uint16_t lnk_s[K::MAXP];     // new triangle whose boundary edge starts at plane x
+    union {
+        uint16_t lnk_s[K::MAXP];     // new triangle whose boundary edge starts at plane x
+        uint32_t vmk[TP];            // during a search: the vertex slots in use
+    };
     uint16_t lnk_e[K::MAXP];     // new triangle whose boundary edge ends at plane y
     uint32_t stack[K::STACK];
     uint32_t hist[HIST_BINS];  // radial histogram of an overflowing candidate pass
@@ -935,14 +942,49 @@ __device__ __forceinline__ float axis_gap(float q, float lo, float hi, float L, 
     return d;
 }
 
+// a double as a float, truncated, by integer arithmetic (an FP64 conversion runs at 1/64 of the FP32 rate); 0 below
+// the normal floats
+__device__ __forceinline__ float trunc32(float v) { return v; }
+__device__ __forceinline__ float trunc32(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    const uint32_t m = ((hi & 0x7fffffffu) - (896u << 20)) << 3 | lo >> 29;
+    return __uint_as_float((hi & 0x80000000u) | (e <= 896u ? 0u : e >= 1151u ? 0x7f7fffffu : m));
+}
+
+// A bisector with p cuts a vertex v off only when p lies in the ball around v through the site: whether the box [x0, x1]
+// x ... (relative to the site) reaches into the ball of any vertex of the cell, i.e. |v|^2 - |p - v|^2 >= -tol for some
+// v and p (balls widened by the vertices' error bounds).  Far sharper than the support of the cell's box where many
+// points lie just beyond the cell, at two dozen evaluations.
+template <typename CT, int TP>
+__device__ __noinline__ bool ball_reaches(const WarpSmem<CT, TP>& S, float x0, float y0, float z0, float x1, float y1,
+                                          float z1, float tol) {
+    float best = -INFINITY;
+#pragma unroll 1
+    for (int e = 0; e < TP; e++) {
+        unsigned m = S.vmk[e];
+        while (m) {
+            const Vtx<CT> v = S.tv[e * 32 + __ffs(m) - 1];
+            m &= m - 1;
+            const float vx = trunc32(v.x), vy = trunc32(v.y), vz = trunc32(v.z), ev = trunc32(v.ev);
+            const float dx = fmaxf(fmaxf(x0 - vx, vx - x1), 0.f), dy = fmaxf(fmaxf(y0 - vy, vy - y1), 0.f),
+                        dz = fmaxf(fmaxf(z0 - vz, vz - z1), 0.f);
+            const float b = (vx * vx + vy * vy + vz * vz) - (dx * dx + dy * dy + dz * dz) +
+                            4.f * ev * (fabsf(vx) + fabsf(vy) + fabsf(vz) + ev);
+            best = fmaxf(best, b);
+        }
+    }
+    return best >= -tol;
+}
+
 // Collect sorted indices j != self with rlo2 <= |d|^2 < rhi2 (the same |d|^2 as the clipping loop).
 // Every hit is also counted in a radial histogram of |d|^2 over [rlo2, rhi2) (HIST_BINS bins), so that an
 // overflowing pass can pick a smaller rhi2 that fits.  Returns the count (which may exceed the capacity: only the
 // first Cap::CAND are stored) or -2 on stack overflow.
-template <typename P, typename CT, int TP>
+template <typename P, typename CT, int TP, bool BALLS>
 __device__ int collect(WarpSmem<CT, TP>& S, const P* spos, int64_t N, const Geometry& g, const Tree& t, uint32_t self,
                        const P& pi, CT rlo2, CT rhi2, const float* bmin, const float* bmax, int64_t slo,
-                       int64_t shi) {
+                       int64_t shi, bool balls) {
     const unsigned lane = lane_id(), lt = lanemask_lt();
     for (int k = (int)lane; k < HIST_BINS; k += 32) S.hist[k] = 0u;
     __syncwarp();
@@ -998,6 +1040,7 @@ __device__ int collect(WarpSmem<CT, TP>& S, const P* spos, int64_t N, const Geom
                     float fx = (float)dx, fy = (float)dy, fz = (float)dz;
                     float sg = supp_g(fx, bmin[0], bmax[0]) + supp_g(fy, bmin[1], bmax[1]) + supp_g(fz, bmin[2], bmax[2]);
                     if (sg < -stol) hit = false;
+                    if (BALLS && hit && balls) hit = ball_reaches<CT, TP>(S, fx, fy, fz, fx, fy, fz, stol);
                 }
                 // order-preserving key: d2 >= 0 so its float bits sort like the value; FP64 values are
                 // rounded down so that a key never exceeds the |d|^2 it stands for
@@ -1041,6 +1084,10 @@ __device__ int collect(WarpSmem<CT, TP>& S, const P* spos, int64_t N, const Geom
                     float sy = supp_axis(qy, lo.y - slack, hi.y + slack, g.Lf[1], per, bmin[1], bmax[1]);
                     float sz = supp_axis(qz, lo.z - slack, hi.z + slack, g.Lf[2], per, bmin[2], bmax[2]);
                     if (sx + sy + sz < -stol) hit = false;
+                    // (a search that meets no periodic image)
+                    if (BALLS && hit && balls && !per)
+                        hit = ball_reaches<CT, TP>(S, lo.x - qx - slack, lo.y - qy - slack, lo.z - qz - slack,
+                                                   hi.x - qx + slack, hi.y - qy + slack, hi.z - qz + slack, stol);
                 }
             }
             unsigned m = __ballot_sync(0xffffffffu, hit);
@@ -1150,7 +1197,7 @@ __device__ __forceinline__ void test_slots(const WarpSmem<CT, TP>& S, unsigned* 
     for (int q = 0; q < TP; q++) masks[q] = 0u;
 }
 
-template <typename P, typename CT, bool EXACT, int TP, bool SETS>
+template <typename P, typename CT, bool EXACT, int TP, bool SETS, bool BALLS>
 __device__ int do_cell(WarpSmem<CT, TP>& S, const ClipArgs& A, uint32_t self, double* xws,
                                     CellCounters& cc, bool small_box) {
     const P* spos = (const P*)A.spos;
@@ -1290,9 +1337,17 @@ __device__ int do_cell(WarpSmem<CT, TP>& S, const ClipArgs& A, uint32_t self, do
         cc.n_passes++;
         if (rhi2 > cap2) rhi2 = cap2;
         int cnt = -1;
+        const bool balls = BALLS && pass >= (A.warp_list ? 1 : BALL_PASS);
+        if (balls) {
+            if (lane == 0)
+#pragma unroll
+                for (int e = 0; e < TP; e++) S.vmk[e] = C.vm[e];
+            __syncwarp();
+        }
         VT_T0(tc0);
         for (int shrink = 0; shrink < 64; shrink++) {
-            cnt = collect<P, CT, TP>(S, spos, A.N, g, A.tree, self, pi, rlo2, rhi2, bmin, bmax, slo, shi);
+            cnt = collect<P, CT, TP, BALLS>(S, spos, A.N, g, A.tree, self, pi, rlo2, rhi2, bmin, bmax, slo, shi,
+                                         balls);
             cc.n_collect++;
             if (cnt > 0) cc.n_collected += cnt;
             if (cnt == -2) return CAP_STACK;
@@ -1575,7 +1630,7 @@ __device__ int do_cell(WarpSmem<CT, TP>& S, const ClipArgs& A, uint32_t self, do
 // Fast kernels: Cap<4>, CLIP_WARPS warps per block, every cell; cells they cannot finish (an undecided FP64
 // test, an ill-conditioned vertex or a capacity overflow) are appended to the exact list.
 // Exact kernel: Cap<16>, one warp per block, the listed cells, exact predicates.
-template <typename P, typename CT, bool EXACT, int TP, int WPB, bool SETS>
+template <typename P, typename CT, bool EXACT, int TP, int WPB, bool SETS, bool BALLS>
 __global__ void __launch_bounds__(WPB * 32) k_clip(ClipArgs A) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int w = threadIdx.x >> 5;
@@ -1589,10 +1644,11 @@ __global__ void __launch_bounds__(WPB * 32) k_clip(ClipArgs A) {
     const uint32_t total = EXACT ? 0u : (uint32_t)A.N;
     for (;;) {
         uint32_t base = 0;
-        const unsigned chunk = EXACT ? 1u : (unsigned)CHUNK;
+        const bool listed = !EXACT && A.warp_list != nullptr;
+        // (a list holds the cells other kernels gave up: the widest ones, one at a time)
+        const unsigned chunk = EXACT || listed ? 1u : (unsigned)CHUNK;
         if (lane == 0) base = atomicAdd(EXACT ? &A.st->work_next_exact : &A.st->work_next, chunk);
         base = __shfl_sync(0xffffffffu, base, 0);
-        const bool listed = !EXACT && A.warp_list != nullptr;
         uint32_t lim = EXACT ? *((volatile unsigned*)&A.st->n_exact_cells)
                              : listed ? *((volatile unsigned*)&A.st->n_warp_cells) : total;
         if (base >= lim) break;
@@ -1605,7 +1661,7 @@ __global__ void __launch_bounds__(WPB * 32) k_clip(ClipArgs A) {
             int rc = 0;
 #pragma unroll 1
             for (int attempt = 0; attempt < 2; attempt++) {
-                rc = do_cell<P, CT, EXACT, TP, SETS>(S, A, self, xws, cc, !EXACT && attempt == 0);
+                rc = do_cell<P, CT, EXACT, TP, SETS, BALLS>(S, A, self, xws, cc, !EXACT && attempt == 0);
                 if (rc != RC_RETRY_BOX) break;
             }
             VT_T1(cc, 5, tall);
@@ -1665,7 +1721,7 @@ __global__ void __launch_bounds__(WPB * 32) k_clip(ClipArgs A) {
 }  // namespace vt
 
 namespace vt {
-template <typename P, typename CT, bool EXACT, bool SETS>
+template <typename P, typename CT, bool EXACT, bool SETS, bool BALLS>
 static void launch_one_t(const ClipArgs& a, int sm_count, cudaStream_t s) {
     constexpr int TP = EXACT ? 16 : 4;
     constexpr int WPB = EXACT ? 1 : CLIP_WARPS;
@@ -1677,18 +1733,25 @@ static void launch_one_t(const ClipArgs& a, int sm_count, cudaStream_t s) {
     cudaGetDevice(&dev);
     int per_sm = (dev >= 0 && dev < 64) ? per_sm_dev[dev] : 0;
     if (per_sm == 0) {
-        cudaFuncSetAttribute(k_clip<P, CT, EXACT, TP, WPB, SETS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_clip<P, CT, EXACT, TP, WPB, SETS>, WPB * 32, smem);
+        cudaFuncSetAttribute(k_clip<P, CT, EXACT, TP, WPB, SETS, BALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_clip<P, CT, EXACT, TP, WPB, SETS, BALLS>, WPB * 32, smem);
         if (per_sm < 1) per_sm = 1;
         if (dev >= 0 && dev < 64) per_sm_dev[dev] = per_sm;
     }
     int blocks = sm_count * per_sm;
     if (EXACT) blocks = a.xws_warps < blocks ? a.xws_warps : blocks;
-    k_clip<P, CT, EXACT, TP, WPB, SETS><<<blocks, WPB * 32, smem, s>>>(a);
+    k_clip<P, CT, EXACT, TP, WPB, SETS, BALLS><<<blocks, WPB * 32, smem, s>>>(a);
 }
 template <typename P, typename CT, bool EXACT>
 static void launch_one(const ClipArgs& a, int sm_count, cudaStream_t s) {
-    if (a.sset) launch_one_t<P, CT, EXACT, true>(a, sm_count, s);
-    else launch_one_t<P, CT, EXACT, false>(a, sm_count, s);
+    // searches against the vertices' balls: for listed cells and larger sets.  Below 8192 particles no halo holds enough
+    // points to make a cell's search long, and the extra code costs 3 % (505 -> 521 us at 1000 uniform points)
+    if (EXACT || (!a.warp_list && a.N <= 8192)) {
+        if (a.sset) launch_one_t<P, CT, EXACT, true, false>(a, sm_count, s);
+        else launch_one_t<P, CT, EXACT, false, false>(a, sm_count, s);
+    } else {
+        if (a.sset) launch_one_t<P, CT, EXACT, true, !EXACT>(a, sm_count, s);
+        else launch_one_t<P, CT, EXACT, false, !EXACT>(a, sm_count, s);
+    }
 }
 }  // namespace vt
