@@ -72,11 +72,12 @@ typedef struct vt_params {
     int k_target;   /* particles aimed for in a cell's first candidate pass (default 24) */
     int max_passes; /* candidate radius passes per cell before VT_ERR_SECURITY (default 1000) */
     int face_pool;  /* facet records reserved per particle (default 24; grown on demand) */
-    int threads_per_cell; /* VT_FILTER32 only: 32 = one warp per cell (default; 0 means 32); 1 = one thread
-                             per cell first, 32 cells of a search-tree bucket per warp; 4 or 8 = that many
-                             lanes per cell first (8 or 4 cells per warp, the cell in shared memory, the
-                             side tests split by vertex); in each case the cells the first kernel cannot
-                             finish are then taken by a warp each (same cells) */
+    int threads_per_cell; /* VT_FILTER32 only: 0 = the library's choice (default): 4 from 65,536 particles on (32
+                             where the device has no room for their memory), else 32; 32 = one warp per cell; 4 or
+                             8 = that many lanes per cell (8 or 4 cells per warp); 1 = one thread per cell, 32 cells
+                             of a search-tree bucket per warp; but for 32, the cells the first kernels cannot finish
+                             are then taken by a warp each (same cells; 4, 8 and 32 give the same bits).  4 and 8
+                             add 2.6 KB of workspace per particle, up to 5.4 GB in all */
     int reserved[3]; /* [0]: candidate pass sizing, 0 = radius doubling up to 2R, 1 = also limited (default)
                         by the density seen so far; others must be 0 */
 } vt_params;
@@ -99,7 +100,7 @@ typedef struct vt_stats {
     double t_clip_ms;         /* device time of vt_build's clipping kernels, last attempt (CUDA events) */
     int64_t reserved[3];      /* diagnostics: [0] internal detail of device_error, [1] candidate collections,
                                  [2] candidates collected */
-    int64_t n_handed_over;    /* FP32 filter: cells the thread-per-cell kernel handed to the warp-per-cell kernel */
+    int64_t n_handed_over;    /* FP32 filter: cells the thread-per-cell or lane-group kernels handed to the warp kernel */
     int64_t n_bucket_passes;  /* FP32 filter: radius passes of the thread-per-cell kernel, summed over buckets */
     int64_t n_grid_failed;    /* cell/voxel parts the last vt_grid_density_volume could not compute (0 normally) */
 } vt_stats;
@@ -201,7 +202,7 @@ int vt_probe_fp64_tflops(double *tflops, void *stream);
  *   boxes    host [n_sets][6]: lo x,y,z then hi x,y,z of each set's box; the
  *            cells of a set are clipped by its box walls (no periodic images)
  *   set_k    host [n_sets] k_target of each set, or NULL (p's k_target)
- *   set_tpc  host [n_sets] threads_per_cell of each set (1, 4, 8 or 32; 0 means 32),
+ *   set_tpc  host [n_sets] threads_per_cell of each set (1, 4, 8 or 32; 0: the library's choice),
  *            or NULL (p's threads_per_cell); see vt_autotune_batched
  *   p, stream  as for vt_build
  * A particle's neighbours are particles of its own set only.  The handle
@@ -390,7 +391,8 @@ int vt_last_error_detail(int *particle);
 /*
  * vt_debug_fail_alloc -- fault injection for tests (no counterpart in the paper): the nth device allocation
  * that vt_build or vt_build_batched makes for a handle's workspace from now on (counting from 1) fails as if
- * cudaMalloc had run out of memory, and the call returns VT_ERR_OOM after freeing what it had allocated.  The
+ * cudaMalloc had run out of memory, and the call returns VT_ERR_OOM after freeing what it had allocated (where the
+ * library chose lane groups by itself, a failure of their memory makes it build with a warp per cell instead).  The
  * hook fires once and disarms; nth <= 0 disarms it.  Process-wide (all host threads, all devices); returns the
  * previous setting (0 if the hook was disarmed or has fired).  Touches no device.
  */

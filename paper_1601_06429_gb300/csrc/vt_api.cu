@@ -140,10 +140,10 @@ void free_handle(vt_handle h) {
     if (!h) return;
     for (int k = 0; k < 4; k++)
         if (h->ev[k]) cudaEventDestroy(h->ev[k]);
-    void* ptrs[] = {h->spos, h->perm, h->inv, h->tree_mem, h->cell, h->face_start, h->face_count, h->cstat, h->rad,
+    void* ptrs[] = {h->spos, h->spos4, h->perm, h->inv, h->tree_mem, h->cell, h->face_start, h->face_count, h->cstat, h->rad,
                     h->exact_list, h->dens_sorted, h->faces, h->xws, h->tmp, h->nbr_off_cache, h->dstat,
                     h->keys, h->keys_alt, h->vals_alt, h->cnt_in, h->sset, h->sgeo, h->soff, h->set_in, h->warp_list,
-                    h->set_cfg, h->gacc, h->gretry, h->gcnt};
+                    h->set_cfg, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_ctr, h->gacc, h->gretry, h->gcnt};
     for (void* p : ptrs)
         if (p) pool_free(p, h->stream);
     map_give(h->smap);
@@ -219,8 +219,11 @@ ClipArgs clip_args(vt_handle h) {
     a.sgeo = h->sgeo;
     a.soff = h->soff;
     // another kernel first (thread per cell, or a lane group) when some cell takes a mode other than the warp's
-    const bool thread_first = (h->modes & ~1) != 0;
-    a.list_given = h->n_owned < h->N;
+    const bool thread_first = (h->modes & ~1) != 0, owned = h->n_owned < h->N;
+    a.list_given = owned && !thread_first;
+    a.n_own = h->n_owned;
+    a.perm = h->perm;
+    a.spos4 = h->dtype == VT_F32 ? (const float4*)h->spos : h->spos4;
     a.warp_list = (thread_first || a.list_given) ? h->warp_list : nullptr;
     a.set_cfg = h->set_cfg;
     a.tpc_mode = h->prm.precision == VT_FILTER32 ? tpc_mode_of(h->prm.threads_per_cell) : 0;
@@ -237,8 +240,20 @@ int enqueue_owned(vt_handle h) {
     int rc = cuda_rc(cudaMemsetAsync(h->cell, 0, (size_t)h->N * sizeof(CellOut), s));
     if (!rc) rc = cuda_rc(cudaMemsetAsync(h->face_count, 0, (size_t)h->N * sizeof(uint16_t), s));
     if (!rc) rc = cuda_rc(cudaMemsetAsync(h->rad, 0, (size_t)h->N * sizeof(float), s));
-    if (!rc) h->n_launches += launch_owned_list(h->inv, h->n_owned, h->warp_list, h->dstat, s);
+    // (the lane-group kernels tell the owned cells by their input rows)
+    if (!rc && (h->modes & ~1) == 0) h->n_launches += launch_owned_list(h->inv, h->n_owned, h->warp_list, h->dstat, s);
     return rc;
+}
+
+GroupBuf group_buf(vt_handle h) {
+    GroupBuf b;
+    b.stat = h->g_stat;
+    b.hdr = (GHdr*)h->g_hdr;
+    b.list = h->g_list;
+    b.state = h->g_state;
+    b.ctr = h->g_ctr;
+    b.chunk = group_chunk(h->N);
+    return b;
 }
 
 int run_clip(vt_handle h) {
@@ -250,8 +265,9 @@ int run_clip(vt_handle h) {
         int rc = enqueue_owned(h);
         if (rc) return rc;
         ClipArgs a = clip_args(h);
+        const GroupBuf gb = group_buf(h);
         cudaEventRecord(h->ev[2], s);
-        h->n_launches += launch_clip(a, h->dtype, h->precision, h->sm_count, s);
+        h->n_launches += launch_clip(a, &gb, h->dtype, h->precision, h->sm_count, s);
         h->n_launches += launch_clip_exact(a, h->dtype, h->sm_count, s);
         cudaEventRecord(h->ev[3], s);
         rc = cuda_rc(cudaGetLastError());
@@ -303,12 +319,20 @@ int vt_default_params(vt_params* p) {
 
 namespace {
 
-int check_params(const vt_params* p, vt_params& prm) {
+// Threads per cell where the caller leaves the choice to the library (0).  FP32 filter: 4 lanes a cell from 65,536
+// particles on, where the chip has enough cells for 8 of them to share a warp; clipping at 32,768 / 65,536 / 2,097,152
+// uniform points takes 1.94 / 3.48 / 114.5 ms by a warp a cell and 1.65 / 2.47 / 40.2 ms by 4 lanes, at 32,768 /
+// 65,536 / 150,000 / 2,097,152 clustered points 3.21 / 6.17 / 12.4 / 128 ms and 4.84 / 6.76 / 8.8 / 61.4 ms (8 lanes
+// are slower than 4 at every size).
+constexpr int64_t GROUP_MIN_N = 65536;
+int default_tpc(int precision, int64_t N) { return precision == VT_FILTER32 && N >= GROUP_MIN_N ? 4 : 32; }
+
+int check_params(const vt_params* p, vt_params& prm, int64_t N) {
     vt_default_params(&prm);
     if (p) prm = *p;
     if (prm.precision != VT_PLAIN64 && prm.precision != VT_FILTER32) return VT_ERR_INVALID;
     if (prm.reserved[0] < 0 || prm.reserved[0] > 1 || prm.reserved[1] || prm.reserved[2]) return VT_ERR_INVALID;
-    if (prm.threads_per_cell == 0) prm.threads_per_cell = 32;
+    if (prm.threads_per_cell == 0) prm.threads_per_cell = default_tpc(prm.precision, N);
     if (tpc_mode_of(prm.threads_per_cell) < 0) return VT_ERR_INVALID;
     if (prm.k_target < 8 || prm.k_target > 120 || prm.max_passes < 1 || prm.max_passes > 100000 || prm.face_pool < 1 ||
         prm.face_pool > 128)
@@ -354,15 +378,16 @@ void enqueue_sort_tree(vt_handle h, const void* pos, const void* mass) {
         h->n_launches += launch_key(pos, h->dtype, N, h->geo, h->keys, h->perm, h->dstat, s);
         h->n_launches += radix_sort(h->keys, h->perm, h->keys_alt, h->vals_alt, N, 48, h->tmp, s);
     }
-    h->n_launches += launch_gather(pos, mass, h->dtype, h->perm, N, h->spos, h->inv, s);
+    h->n_launches += launch_gather(pos, mass, h->dtype, h->perm, N, h->spos, h->spos4, h->inv, s);
     h->n_launches += launch_tree(h->spos, h->dtype, N, h->tree, s);
 }
 
 // Shared by vt_build (n_sets == 0: one set, geometry `geo`) and vt_build_batched (n_sets >= 1: the host
-// tables set_off [n_sets+1] and sgeo [n_sets]).
+// tables set_off [n_sets+1] and sgeo [n_sets]).  chosen: the threads per cell are the library's choice, so that a
+// device without room for the lane-group kernels' memory falls back to a warp a cell.
 int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int64_t N, const Geometry& geo,
-               int n_sets, const int64_t* set_off, const Geometry* sgeo_host, const int32_t* cfg_host,
-               const vt_params& prm, void* stream, int64_t n_owned = -1) {
+               int n_sets, const int64_t* set_off, const Geometry* sgeo_host, int32_t* cfg_host,
+               const vt_params& prm, bool chosen, void* stream, int64_t n_owned = -1) {
     vt_handle h = new (std::nothrow) vt_handle_s;
     if (!h) return VT_ERR_OOM;
     memset(h, 0, sizeof(*h));
@@ -378,6 +403,14 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (h->sm_count <= 0) h->sm_count = 1;
+
+    // the threads-per-cell modes present: each set's, or the handle's
+    if (cfg_host) {
+        for (int k = 0; k < n_sets; k++)
+            if (set_off[k + 1] > set_off[k]) h->modes |= 1 << ((cfg_host[k] >> 16) & 3);
+    } else {
+        h->modes = 1 << (prm.precision == VT_FILTER32 ? tpc_mode_of(prm.threads_per_cell) : 0);
+    }
 
     Alloc A;
     A.s = h->stream;
@@ -419,19 +452,37 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
         h->soff = A.get<int64_t>(n_sets + 1);
         if (cfg_host) h->set_cfg = A.get<int32_t>(n_sets);
     }
-    // the threads-per-cell modes present: each set's, or the handle's
-    if (cfg_host) {
-        for (int k = 0; k < n_sets; k++)
-            if (set_off[k + 1] > set_off[k]) h->modes |= 1 << ((cfg_host[k] >> 16) & 3);
-    } else {
-        h->modes = 1 << (prm.precision == VT_FILTER32 ? tpc_mode_of(prm.threads_per_cell) : 0);
-    }
     for (int k = 0; k < 4; k++)
         if (cudaEventCreate(&h->ev[k]) != cudaSuccess) {
             cudaGetLastError();
             h->ev[k] = nullptr;
             A.failed = true;
         }
+    if (!A.failed && (h->modes & 12)) {
+        // last, so that what fits without the lane-group kernels' memory still fits
+        const size_t m = group_chunk(N);
+        if (dtype == VT_F64) h->spos4 = A.get<float4>(N);
+        h->g_stat = A.get<uint8_t>(m);
+        h->g_hdr = A.get<GHdr>(m);
+        h->g_list = A.get<uint32_t>(m * GROUP_CAND);
+        h->g_state = A.get<unsigned char>(m * GROUP_STATE);
+        h->g_ctr = A.get<uint32_t>(group_counters(N));
+        if (A.failed && chosen) {
+            void* g[] = {h->spos4, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_ctr};
+            for (void* p : g)
+                if (p) pool_free(p, h->stream);
+            h->spos4 = nullptr;
+            h->g_stat = nullptr;
+            h->g_hdr = nullptr;
+            h->g_list = nullptr;
+            h->g_state = nullptr;
+            h->g_ctr = nullptr;
+            h->modes = 1;
+            h->prm.threads_per_cell = 32;
+            for (int k = 0; cfg_host && k < n_sets; k++) cfg_host[k] &= 0xffff;
+            A.failed = false;
+        }
+    }
     if (A.failed) {
         free_handle(h);
         return VT_ERR_OOM;
@@ -489,12 +540,12 @@ int vt_build(vt_handle* out, const void* pos, int dtype, const void* mass, int64
     if (!pos || !box_lo || !box_hi || N < 1 || N > 0x7FFFFFFF / 2) return VT_ERR_INVALID;
     if (dtype != VT_F32 && dtype != VT_F64) return VT_ERR_INVALID;
     vt_params prm;
-    int rc = check_params(p, prm);
+    int rc = check_params(p, prm, N);
     if (rc) return rc;
     Geometry geo;
     rc = make_geometry(box_lo, box_hi, periodic, prm.precision, geo);
     if (rc) return rc;
-    return build_impl(out, pos, dtype, mass, N, geo, 0, nullptr, nullptr, nullptr, prm, stream);
+    return build_impl(out, pos, dtype, mass, N, geo, 0, nullptr, nullptr, nullptr, prm, !p || !p->threads_per_cell, stream);
 }
 
 int vt_build_owned(vt_handle* out, const void* pos, int dtype, const void* mass, int64_t N, int64_t n_owned,
@@ -504,13 +555,14 @@ int vt_build_owned(vt_handle* out, const void* pos, int dtype, const void* mass,
     if (!pos || !box_lo || !box_hi || N < 1 || N > 0x7FFFFFFF / 2 || n_owned < 1 || n_owned > N) return VT_ERR_INVALID;
     if (dtype != VT_F32 && dtype != VT_F64) return VT_ERR_INVALID;
     vt_params prm;
-    int rc = check_params(p, prm);
+    int rc = check_params(p, prm, N);
     if (rc) return rc;
-    prm.threads_per_cell = 32;  // the listed cells go to the warp kernel
+    // the listed cells go to the lane-group kernel by the library's choice, to the warp kernel otherwise
+    prm.threads_per_cell = p && p->threads_per_cell ? 32 : prm.threads_per_cell;
     Geometry geo;
     rc = make_geometry(box_lo, box_hi, periodic, prm.precision, geo);
     if (rc) return rc;
-    return build_impl(out, pos, dtype, mass, N, geo, 0, nullptr, nullptr, nullptr, prm, stream, n_owned);
+    return build_impl(out, pos, dtype, mass, N, geo, 0, nullptr, nullptr, nullptr, prm, true, stream, n_owned);
 }
 
 int vt_build_batched(vt_handle* out, const void* pos, int dtype, const void* mass, const int64_t* set_off, int n_sets,
@@ -526,7 +578,7 @@ int vt_build_batched(vt_handle* out, const void* pos, int dtype, const void* mas
     const int64_t N = set_off[n_sets];
     if (N < 1 || N > 0x7FFFFFFF / 2) return VT_ERR_INVALID;
     vt_params prm;
-    int rc = check_params(p, prm);
+    int rc = check_params(p, prm, N);
     if (rc) return rc;
     Geometry* sg = new (std::nothrow) Geometry[n_sets];
     int32_t* cfg = (set_k || set_tpc) ? new (std::nothrow) int32_t[n_sets] : nullptr;
@@ -538,12 +590,15 @@ int vt_build_batched(vt_handle* out, const void* pos, int dtype, const void* mas
     for (int k = 0; k < n_sets && !rc; k++) rc = make_geometry(boxes + 6 * k, boxes + 6 * k + 3, 0, prm.precision, sg[k]);
     for (int k = 0; cfg && k < n_sets && !rc; k++) {
         const int kt = set_k ? set_k[k] : prm.k_target;
-        const int tpc = set_tpc ? (set_tpc[k] ? set_tpc[k] : 32) : prm.threads_per_cell;
+        const int tpc = set_tpc ? (set_tpc[k] ? set_tpc[k] : default_tpc(prm.precision, N)) : prm.threads_per_cell;
         if (kt < 8 || kt > 120 || tpc_mode_of(tpc) < 0) rc = VT_ERR_INVALID;
         // the thread-per-cell and lane-group kernels exist for the FP32 filter only
         cfg[k] = kt | (prm.precision == VT_FILTER32 && tpc_mode_of(tpc) > 0 ? tpc_mode_of(tpc) << 16 : 0);
     }
-    if (!rc) rc = build_impl(out, pos, dtype, mass, N, sg[0], n_sets, set_off, sg, cfg, prm, stream);
+    // the library's choice: no set asks for lane groups or one thread itself
+    bool chosen = !p || !p->threads_per_cell || p->threads_per_cell == 32;
+    for (int k = 0; set_tpc && k < n_sets; k++) chosen = chosen && (set_tpc[k] == 0 || set_tpc[k] == 32);
+    if (!rc) rc = build_impl(out, pos, dtype, mass, N, sg[0], n_sets, set_off, sg, cfg, prm, chosen, stream);
     delete[] sg;
     delete[] cfg;
     return rc;
@@ -558,7 +613,7 @@ int vt_autotune_batched(const void* pos, int dtype, const int64_t* set_off, int 
         if (set_off[k + 1] < set_off[k]) return VT_ERR_INVALID;
     if (set_off[n_sets] < 1 || set_off[n_sets] > 0x7FFFFFFF / 2) return VT_ERR_INVALID;
     vt_params prm;
-    int rc = check_params(p, prm);
+    int rc = check_params(p, prm, set_off[n_sets]);
     if (rc) return rc;
     if (sample <= 0) sample = 262144;
     if (sample < 1024) sample = 1024;
@@ -622,7 +677,7 @@ int vt_autotune_batched(const void* pos, int dtype, const int64_t* set_off, int 
                 t.threads_per_cell = tpcs[trial / 5];
             }
             vt_handle h = nullptr;
-            const int e = build_impl(&h, buf, dtype, nullptr, tot, sg[0], np, soff, sg, nullptr, t, stream);
+            const int e = build_impl(&h, buf, dtype, nullptr, tot, sg[0], np, soff, sg, nullptr, t, false, stream);
             if (e) {
                 last_err = e;
                 continue;
@@ -663,7 +718,8 @@ int vt_rebuild(vt_handle h, const void* pos, const void* mass) {
     rc = enqueue_owned(h);
     if (rc) return rc;
     ClipArgs a = clip_args(h);
-    h->n_launches += launch_clip(a, h->dtype, h->precision, h->sm_count, s);
+    const GroupBuf gb = group_buf(h);
+    h->n_launches += launch_clip(a, &gb, h->dtype, h->precision, h->sm_count, s);
     h->n_launches += launch_clip_exact(a, h->dtype, h->sm_count, s);
     h->dens_ready = 0;
     h->faces_on_device = 1;

@@ -103,6 +103,7 @@ struct vt_handle_s {
     int modes;          // threads-per-cell modes present among the cells (bit m: mode m, see ClipArgs)
     // sorted particles
     void* spos;         // float4 (f32) or double4-like 4 doubles (f64): x,y,z,m
+    float4* spos4;      // FP32 copy of FP64 positions (lane-group kernels only)
     uint32_t* perm;     // sorted -> input index
     uint32_t* inv;      // input -> sorted index
     // search tree
@@ -128,6 +129,12 @@ struct vt_handle_s {
     // exact workspace (per warp of the exact kernel)
     double* xws;
     int xws_warps;
+    // the lane-group kernels' memory (modes that use them only)
+    uint8_t* g_stat;
+    void* g_hdr;
+    uint32_t* g_list;
+    unsigned char* g_state;
+    uint32_t* g_ctr;
     // scratch for sort / scans
     void* tmp;
     size_t tmp_bytes;

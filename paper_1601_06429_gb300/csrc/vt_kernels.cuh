@@ -21,7 +21,7 @@ int radix_sort(uint64_t* key, uint32_t* val, uint64_t* key_alt, uint32_t* val_al
 int launch_key(const void* pos, int dtype, int64_t N, const Geometry& g, uint64_t* key, uint32_t* idx, DevStatus* st,
                 cudaStream_t s);
 int launch_gather(const void* pos, const void* mass, int dtype, const uint32_t* perm, int64_t N, void* spos,
-                   uint32_t* inv, cudaStream_t s);
+                   float4* spos4, uint32_t* inv, cudaStream_t s);
 int launch_key_batched(const void* pos, int dtype, int64_t N, const Geometry* sgeo, const uint32_t* setid,
                        uint64_t* key, uint32_t* idx, DevStatus* st, cudaStream_t s);
 int launch_set_ids(const int64_t* soff, int n_sets, int64_t N, uint32_t* setid, cudaStream_t s);
@@ -67,13 +67,47 @@ struct ClipArgs {
     // list_given: warp_list already holds the cells to compute (st->n_warp_cells of them; the other particles
     // are candidates only) and no thread-per-cell kernel runs
     int list_given;
+    // the lane-group kernels compute the cells of input rows [0, n_own) only (N: all), told by perm (sorted -> input)
+    int64_t n_own;
+    const uint32_t* perm;
+    // the sorted positions in FP32 for its search (spos itself for FP32 positions)
+    const float4* spos4;
     // per-cell radius (sorted order): an upper bound of the largest vertex distance of the final cell, or NULL
     float* rad;
 };
-int launch_clip(const ClipArgs& a, int dtype, int precision, int sm_count, cudaStream_t s);
+// The lane-group kernels' memory (vt_clip_group.cu): per cell of a chunk its status, header, candidate list and the
+// state kept between radius passes (2.2 KB a cell; chunks of at most GROUP_CHUNK cells), and the queue counters of
+// every launch.
+constexpr int GROUP_CAND = 96;
+constexpr int GROUP_NT = 64, GROUP_NP = 40;  // vertex slots and planes of a cell
+constexpr int GROUP_STATE = (GROUP_NT * 20 + GROUP_NP * 21 + 15) / 16 * 16;
+constexpr int GROUP_PASSES = 8;
+constexpr uint32_t GROUP_CHUNK = 1u << 21;
+struct GHdr {
+    float rlo2, rhi2, B, R2, cap2;            // range of |d|^2 of the pass, start box, squared radius, widest search
+    float bx0, by0, bz0, bx1, by1, bz1;       // box around the vertices
+    uint32_t vlo, vhi, n, meta;               // slots in use; candidates | cuts so far << 16; planes | start walls << 8 | FP64 << 16 | passes << 24
+    float first2;                             // squared first radius
+};
+struct GroupBuf {
+    uint8_t* stat;         // wants a pass
+    GHdr* hdr;
+    uint32_t* list;        // [GROUP_CAND] a cell, in order of distance
+    unsigned char* state;  // [GROUP_STATE] a cell
+    uint32_t* ctr;         // [group_counters(N)], zero before the launches
+    uint32_t chunk;        // cells of a chunk (a multiple of 32)
+};
+inline uint32_t group_chunk(int64_t N) {
+    const int64_t n = (N + 31) / 32 * 32;
+    return n < (int64_t)GROUP_CHUNK ? (uint32_t)n : GROUP_CHUNK;
+}
+inline size_t group_counters(int64_t N) {
+    return 2 * 2 * (size_t)GROUP_PASSES * (size_t)((N + group_chunk(N) - 1) / group_chunk(N));
+}
+int launch_clip(const ClipArgs& a, const GroupBuf* gb, int dtype, int precision, int sm_count, cudaStream_t s);
 int launch_clip_exact(const ClipArgs& a, int dtype, int sm_count, cudaStream_t s);
 int launch_clip_thread(const ClipArgs& a, int dtype, int sm_count, cudaStream_t s);
-int launch_clip_group(const ClipArgs& a, int dtype, int lanes, int sm_count, cudaStream_t s);
+int launch_clip_group(const ClipArgs& a, const GroupBuf& b, int dtype, int lanes, int sm_count, cudaStream_t s);
 int launch_fma_probe(int blocks, int iters, float* sink, cudaStream_t s);
 int launch_fma_probe64(int blocks, int iters, double* sink, cudaStream_t s);
 int launch_cvt_weighted(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,

@@ -145,7 +145,7 @@ extern "C" int vt_volumes_noalloc(const void* pos, int dtype, int64_t N, const d
     if (rc) return rc;
     launch_key(pos, dtype, N, geo, keys, perm, dstat, s);
     radix_sort(keys, perm, keys_alt, vals_alt, N, 48, tmp, s);
-    launch_gather(pos, nullptr, dtype, perm, N, spos, inv, s);
+    launch_gather(pos, nullptr, dtype, perm, N, spos, nullptr, inv, s);
     launch_tree(spos, dtype, N, tree, s);
     ClipArgs a;
     memset(&a, 0, sizeof(a));
@@ -167,7 +167,7 @@ extern "C" int vt_volumes_noalloc(const void* pos, int dtype, int64_t N, const d
     a.xws = xws;
     a.xws_warps = kExactWarps;
     a.warp_list = nullptr;  // the warp-per-cell kernel on every cell, as vt_build's default
-    launch_clip(a, dtype, VT_FILTER32, sms, s);
+    launch_clip(a, nullptr, dtype, VT_FILTER32, sms, s);
     launch_clip_exact(a, dtype, sms, s);
     rc = rc_of(cudaGetLastError());
     if (rc) return rc;

@@ -375,9 +375,10 @@ int radix_sort(uint64_t* key, uint32_t* val, uint64_t* key_alt, uint32_t* val_al
 }
 
 // ---------------------------------------------------------------- gather
+// spos4 (or NULL): the FP32 copy of FP64 positions that the lane-group kernel's search reads
 template <typename T, typename P>
 __global__ void k_gather(const T* __restrict__ pos, const T* __restrict__ mass, const uint32_t* __restrict__ perm,
-                         int64_t N, P* __restrict__ spos, uint32_t* __restrict__ inv) {
+                         int64_t N, P* __restrict__ spos, float4* __restrict__ spos4, uint32_t* __restrict__ inv) {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= N) return;
     uint32_t i = perm[k];
@@ -387,6 +388,7 @@ __global__ void k_gather(const T* __restrict__ pos, const T* __restrict__ mass, 
     p.z = pos[3 * (int64_t)i + 2];
     p.w = mass ? mass[i] : (T)1;
     spos[k] = p;
+    if (spos4) spos4[k] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.f);
     inv[i] = (uint32_t)k;
 }
 
@@ -404,12 +406,12 @@ int launch_key(const void* pos, int dtype, int64_t N, const Geometry& g, uint64_
 }
 
 int launch_gather(const void* pos, const void* mass, int dtype, const uint32_t* perm, int64_t N, void* spos,
-                  uint32_t* inv, cudaStream_t s) {
+                  float4* spos4, uint32_t* inv, cudaStream_t s) {
     unsigned nb = (unsigned)((N + 255) / 256);
     if (dtype == VT_F32)
-        k_gather<float, float4><<<nb, 256, 0, s>>>((const float*)pos, (const float*)mass, perm, N, (float4*)spos, inv);
+        k_gather<float, float4><<<nb, 256, 0, s>>>((const float*)pos, (const float*)mass, perm, N, (float4*)spos, spos4, inv);
     else
-        k_gather<double, dpt4><<<nb, 256, 0, s>>>((const double*)pos, (const double*)mass, perm, N, (dpt4*)spos, inv);
+        k_gather<double, dpt4><<<nb, 256, 0, s>>>((const double*)pos, (const double*)mass, perm, N, (dpt4*)spos, spos4, inv);
     return 1;
 }
 
