@@ -143,7 +143,7 @@ void free_handle(vt_handle h) {
     void* ptrs[] = {h->spos, h->spos4, h->perm, h->inv, h->tree_mem, h->cell, h->face_start, h->face_count, h->cstat, h->rad,
                     h->exact_list, h->dens_sorted, h->faces, h->xws, h->tmp, h->nbr_off_cache, h->dstat,
                     h->keys, h->keys_alt, h->vals_alt, h->cnt_in, h->sset, h->sgeo, h->soff, h->set_in, h->warp_list,
-                    h->set_cfg, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_ctr, h->gacc, h->gretry, h->gcnt};
+                    h->set_cfg, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_act, h->g_ctr, h->gacc, h->gretry, h->gcnt};
     for (void* p : ptrs)
         if (p) pool_free(p, h->stream);
     map_give(h->smap);
@@ -251,6 +251,7 @@ GroupBuf group_buf(vt_handle h) {
     b.hdr = (GHdr*)h->g_hdr;
     b.list = h->g_list;
     b.state = h->g_state;
+    b.act = h->g_act;
     b.ctr = h->g_ctr;
     b.chunk = group_chunk(h->N);
     return b;
@@ -466,9 +467,10 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
         h->g_hdr = A.get<GHdr>(m);
         h->g_list = A.get<uint32_t>(m * GROUP_CAND);
         h->g_state = A.get<unsigned char>(m * GROUP_STATE);
+        h->g_act = A.get<uint32_t>(2 * m);
         h->g_ctr = A.get<uint32_t>(group_counters(N));
         if (A.failed && chosen) {
-            void* g[] = {h->spos4, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_ctr};
+            void* g[] = {h->spos4, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_act, h->g_ctr};
             for (void* p : g)
                 if (p) pool_free(p, h->stream);
             h->spos4 = nullptr;
@@ -476,6 +478,7 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
             h->g_hdr = nullptr;
             h->g_list = nullptr;
             h->g_state = nullptr;
+            h->g_act = nullptr;
             h->g_ctr = nullptr;
             h->modes = 1;
             h->prm.threads_per_cell = 32;

@@ -42,7 +42,8 @@ constexpr int SWARPS = 4;  // warps per block of the search kernel
 constexpr int GBINS = 64;  // radial bins of the candidate ordering (one byte counter each)
 // from this radius pass on points too are tested against the vertices' balls (nodes from the second pass on): from the
 // second pass on it costs more than the tests it saves (59 against 53 ms at 1,048,576 clustered points)
-constexpr uint32_t SWIDE = 2;
+constexpr uint32_t SWIDE = 3;
+constexpr int GLIST = 3;
 constexpr uint32_t GM_INIT = 1u << 17;  // header: the cell starts (again) from its start box
 constexpr int IDB5 = 6;    // bits of a plane id
 constexpr uint32_t IDM5 = (1u << IDB5) - 1u;
@@ -274,7 +275,8 @@ __device__ __forceinline__ bool ball_hit(const SCell& K, float x0, float y0, flo
 template <typename P, bool SETS, bool FIRST>
 __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_constant__ ClipArgs A,
                                                                  const __grid_constant__ GroupBuf B, uint32_t c0, uint32_t nc,
-                                                                 uint32_t* ctr, uint32_t unit, int mode) {
+                                                                 uint32_t* ctr, uint32_t unit, int mode,
+                                                                 const uint32_t* act_list, const uint32_t* n_act) {
     __shared__ SWarp smem[SWARPS];
     SWarp& S = smem[threadIdx.x >> 5];
     const unsigned lane = lane_id(), lt = lanemask_lt();
@@ -282,15 +284,20 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
     const P* const spos = (const P*)A.spos;
     const bool periodic = SETS ? false : A.geo.periodic != 0;
     unsigned c_coll = 0, c_found = 0;
+    const uint32_t count = act_list ? *n_act : nc;
     for (;;) {
         uint32_t b = 0;
         if (lane == 0) b = atomicAdd(ctr, unit);
         b = __shfl_sync(FULL, b, 0);
-        if (b >= nc) break;
-        // the lanes hold the cells of a bucket; the warp searches for `unit` of them
-        const uint32_t i = (b & ~31u) + lane, self = c0 + i;
-        const bool in = i < nc;
-        bool active = in && i >= b && i < b + unit;
+        if (b >= count) break;
+        // the lanes hold the cells of a bucket and the warp searches for `unit` of them, or the next `unit` listed cells
+        uint32_t i = (b & ~31u) + lane;
+        bool in = i < nc, active = in && i >= b && i < b + unit;
+        if (act_list) {
+            in = active = lane < unit && b + lane < count;
+            i = in ? act_list[b + lane] : 0u;
+        }
+        const uint32_t self = c0 + i;
         uint32_t set = 0, slo = 0, shi = (uint32_t)A.N;
         int k_target = A.k_target;
         const bool mine = active;
@@ -421,6 +428,16 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
                 ulo = __reduce_min_sync(FULL, act ? slo : 0xffffffffu);
                 uhi = __reduce_max_sync(FULL, act ? shi : 0u);
             }
+            // ... and the ball around them: half of the box's leaves lie in its corners
+            const float ucx = 0.5f * (ux0 + ux1), ucy = 0.5f * (uy0 + uy1), ucz = 0.5f * (uz0 + uz1);
+            float ur2 = 0.f;
+            if (act) {
+                const float4 q = S.par[own].q;
+                const float ax = q.x - ucx, ay = q.y - ucy, az = q.z - ucz;
+                ur2 = (sqrtf(ax * ax + ay * ay + az * az) + sqrtf(q.w)) * (1.f + 1e-5f) + 2.f * S.par[own].b0.w;
+                ur2 *= ur2;
+            }
+            ur2 = warp_max<float>(ur2);
             cross = __any_sync(FULL, cross);
             unsigned lost = 0u;  // cells whose search failed
             int n = 0;           // lane c: candidates of cell c
@@ -454,20 +471,28 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
                             lo = A.tree.lo[o]; hi = A.tree.hi[o];
                             hit = lo.x + hx <= ux1 && hi.x + hx >= ux0 && lo.y + hy <= uy1 && hi.y + hy >= uy0 &&
                                   lo.z + hz <= uz1 && hi.z + hz >= uz0;
+                            const float ax = fmaxf(fmaxf(lo.x + hx - ucx, ucx - hi.x - hx), 0.f),
+                                        ay = fmaxf(fmaxf(lo.y + hy - ucy, ucy - hi.y - hy), 0.f),
+                                        az = fmaxf(fmaxf(lo.z + hz - ucz, ucz - hi.z - hz), 0.f);
+                            hit = hit && ax * ax + ay * ay + az * az <= ur2;
                             if (SETS) {
                                 const uint64_t f = (uint64_t)c << (5 * cl);
                                 hit = hit && f < uhi && f + (1ull << (5 * cl)) > ulo;
                             }
                         }
                         if (!FIRST && cl > 1 && __any_sync(FULL, hit)) {
-                            // an inner node of a later pass: some cell's annulus and support must reach it
+                            // an inner node of a later pass: some cell's annulus, support and vertices' balls must reach it
                             bool any = false;
 #pragma unroll 1
                             for (int c2 = 0; c2 < ncell; c2++) {
                                 const SCell& K = S.par[c2];
                                 const float4 q = K.q, a = K.a, b0 = K.b0, b1 = K.b1;
-                                any = any || node_may_cut(lo.x + hx - q.x, lo.y + hy - q.y, lo.z + hz - q.z, hi.x + hx - q.x,
-                                                          hi.y + hy - q.y, hi.z + hz - q.z, q.w, a, b0, b1);
+                                const float x0 = lo.x + hx - q.x, y0 = lo.y + hy - q.y, z0 = lo.z + hz - q.z, x1 = hi.x + hx - q.x,
+                                            y1 = hi.y + hy - q.y, z1 = hi.z + hz - q.z;
+                                bool may = hit && !any && node_may_cut(x0, y0, z0, x1, y1, z1, q.w, a, b0, b1);
+                                if (may && K.wide && (K.vlo | K.vhi))
+                                    may = ball_hit(K, x0 - b0.w, y0 - b0.w, z0 - b0.w, x1 + b0.w, y1 + b0.w, z1 + b0.w, a.y);
+                                any = any || may;
                             }
                             hit = hit && any;
                         }
@@ -716,7 +741,9 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
 template <typename P, int G, bool SETS>
 __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __grid_constant__ ClipArgs A,
                                                                      const __grid_constant__ GroupBuf B, uint32_t c0, uint32_t nc,
-                                                                     uint32_t* ctr, int last) {
+                                                                     uint32_t* ctr, int last, const uint32_t* act_list,
+                                                                     const uint32_t* n_act, uint32_t* next_list,
+                                                                     uint32_t* n_next) {
     constexpr int W = 32 / G;   // cells per warp
     constexpr int IT = 32 / G;  // planes per lane
     extern __shared__ __align__(16) unsigned char gsmem[];
@@ -742,8 +769,9 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
     int np = 6, nseq = 6, fail = 0;
     unsigned art = 0u, used64 = 0u;
     float R2 = 0.f, bx0 = 0.f, by0 = 0.f, bz0 = 0.f, bx1 = 0.f, by1 = 0.f, bz1 = 0.f;
-    // the warp's part of the queue: cells wbase + (bits of wmask)
-    uint32_t wbase = 0;
+    // the warp's part of the queue: the cells wcell of the lanes in wmask
+    const uint32_t count = act_list ? *n_act : nc;
+    uint32_t wbase = 0, wcell = 0;
     unsigned wmask = 0u;
     bool dry = false;
     unsigned c_cut = 0, c_tested = 0, c_pass = 0, c_fp64 = 0, c_faces = 0, c_maxf = 0;
@@ -784,17 +812,20 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
                     uint32_t b = 0;
                     if (lane == 0) b = atomicAdd(ctr, 32u);
                     wbase = __shfl_sync(FULL, b, 0);
-                    if (wbase >= nc) { dry = true; break; }
-                    wmask = __ballot_sync(FULL, wbase + lane < nc && B.stat[wbase + lane] != 0);
+                    if (wbase >= count) { dry = true; break; }
+                    const bool in = wbase + lane < count;
+                    wcell = !in ? 0u : act_list ? act_list[wbase + lane] : wbase + lane;
+                    wmask = __ballot_sync(FULL, in && B.stat[wcell] != 0);
                     continue;
                 }
                 const int give = min(__popc(need), __popc(wmask));
                 const int rank = __popc(need & ((1u << gsh) - 1u));
-                if (((need >> gsh) & 1u) && rank < give) {
-                    unsigned m = wmask;
+                unsigned m = wmask;
 #pragma unroll 1
-                    for (int k = 0; k < rank; k++) m &= m - 1u;
-                    ci = wbase + (uint32_t)(__ffs(m) - 1);
+                for (int k = 0; k < rank; k++) m &= m - 1u;
+                const uint32_t cell = __shfl_sync(FULL, wcell, m ? __ffs(m) - 1 : 0);
+                if (((need >> gsh) & 1u) && rank < give) {
+                    ci = cell;
                     has = fresh = true;
                 }
 #pragma unroll 1
@@ -1122,14 +1153,14 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
             else if (H.rhi2 >= H.cap2 || pass >= A.max_passes || last) fail = GF_RADIUS;
             else {
                 // the annulus up to 2R, at most twice the radius (policy 1: also no further than the radius that the
-                // density seen so far says holds about 3/4 of a pass's capacity)
+                // density seen so far says holds three times a pass's capacity: the support test leaves fewer)
                 const float nxt = 4.f * R2 * (1.f + 32.f * u);
                 float lim2 = 4.f * H.rhi2;
                 if (A.radius_policy == 1 && nlist > 0) {
                     const float rh = sqrtf(H.rhi2), rl = sqrtf(H.rlo2);
                     const float shell = rh * rh * rh - rl * rl * rl;
                     if (shell > 0.f) {
-                        const float rr = cbrtf(rh * rh * rh + 0.75f * GNC * shell / (float)nlist);
+                        const float rr = cbrtf(rh * rh * rh + 3.f * GNC * shell / (float)nlist);
                         lim2 = fminf(lim2, fmaxf(rr * rr, 1.21f * H.rhi2));
                     }
                 }
@@ -1146,6 +1177,7 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
             }
         }
         const unsigned w64 = gor<G>(used64);
+        bool queue = again;  // the cell's next pass
         if (again) {
             GCell* const K = reinterpret_cast<GCell*>(B.state + (size_t)ci * GROUP_STATE);
             const int hw = vhi ? 64 - __clz(vhi) : 32 - __clz(vlo);
@@ -1215,6 +1247,7 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
                 done = false;
                 if (last || !(H.B < INFINITY) || pass >= A.max_passes) fail = GF_WALL;
                 else {
+                    queue = true;
                     if (r == 0) {
                         H.B = INFINITY;
                         H.meta = ((uint32_t)pass << 24) | GM_INIT | (w64 << 16);
@@ -1417,6 +1450,15 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
             }
             __syncwarp();
         }
+        if (next_list) {
+            const unsigned qm = __ballot_sync(FULL, queue) & lead;
+            if (qm) {
+                unsigned slot = 0;
+                if (lane == 0) slot = atomicAdd(n_next, (unsigned)__popc(qm));
+                slot = __shfl_sync(FULL, slot, 0);
+                if (queue && r == 0) next_list[slot + __popc(qm & ((1u << lane) - 1u))] = ci;
+            }
+        }
         // ---------------------------------------------------------------- cells for the warp kernel
         const bool hand = has && fail != 0;
         const unsigned hm = __ballot_sync(FULL, hand) & lead;
@@ -1464,25 +1506,26 @@ int blocks_per_sm(K kernel, int threads, size_t smem, int* per_sm_dev) {
 }
 
 template <typename P, bool SETS, bool FIRST>
-void launch_search(const ClipArgs& a, const GroupBuf& b, uint32_t c0, uint32_t nc, uint32_t* ctr, int mode, int sm_count,
-                   cudaStream_t s) {
+void launch_search(const ClipArgs& a, const GroupBuf& b, uint32_t c0, uint32_t nc, uint32_t* ctr, int mode,
+                   const uint32_t* act, const uint32_t* n_act, int sm_count, cudaStream_t s) {
     static int per_sm_dev[64] = {0};
     const int per_sm = blocks_per_sm(k_group_search<P, SETS, FIRST>, SWARPS * 32, 0, per_sm_dev);
     const unsigned all = (unsigned)(sm_count * per_sm);
     // cells a warp takes at a time: 32 share what is loaded for a bucket; 8 where 32 would leave the chip short of warps
-    const uint32_t unit = FIRST && nc >= 64u * SWARPS * all ? 32u : 8u;
+    // listed cells one by one: they are the widest, and the slowest search is the launch's time
+    const uint32_t unit = act ? 1u : FIRST && nc >= 64u * SWARPS * all ? 32u : 8u;
     const unsigned most = (nc + unit * SWARPS - 1) / (unit * SWARPS);
-    k_group_search<P, SETS, FIRST><<<most < all ? most : all, SWARPS * 32, 0, s>>>(a, b, c0, nc, ctr, unit, mode);
+    k_group_search<P, SETS, FIRST><<<most < all ? most : all, SWARPS * 32, 0, s>>>(a, b, c0, nc, ctr, unit, mode, act, n_act);
 }
 template <typename P, int G, bool SETS>
-void launch_gclip(const ClipArgs& a, const GroupBuf& b, uint32_t c0, uint32_t nc, uint32_t* ctr, int last, int sm_count,
-                  cudaStream_t s) {
+void launch_gclip(const ClipArgs& a, const GroupBuf& b, uint32_t c0, uint32_t nc, uint32_t* ctr, int last,
+                  const uint32_t* act, const uint32_t* n_act, uint32_t* next, uint32_t* n_next, int sm_count, cudaStream_t s) {
     static int per_sm_dev[64] = {0};
     constexpr int W = 32 / G;
     const size_t smem = W * sizeof(GCell);
     const int per_sm = blocks_per_sm(k_group_clip<P, G, SETS>, 32, smem, per_sm_dev);
     const unsigned most = (nc + W - 1) / W, all = (unsigned)(sm_count * per_sm);
-    k_group_clip<P, G, SETS><<<most < all ? most : all, 32, smem, s>>>(a, b, c0, nc, ctr, last);
+    k_group_clip<P, G, SETS><<<most < all ? most : all, 32, smem, s>>>(a, b, c0, nc, ctr, last, act, n_act, next, n_next);
 }
 
 template <typename P, int G, bool SETS>
@@ -1490,14 +1533,20 @@ int launch_group(const ClipArgs& a, const GroupBuf& b, int sm_count, cudaStream_
     constexpr int MODE = G == 4 ? 2 : 3;
     const uint32_t N = (uint32_t)a.N;
     uint32_t* ctr = b.ctr + (G == 4 ? 0 : group_counters(a.N) / 2);
+    // a pass over few cells costs its latency: handing them over after eight is cheaper until there are many
+    const int passes = a.N < (int64_t)(1 << 20) ? 8 : GROUP_PASSES;
     int n = 0;
     for (uint32_t c0 = 0; c0 < N; c0 += b.chunk) {
         const uint32_t nc = N - c0 < b.chunk ? N - c0 : b.chunk;
-        for (int p = 0; p < GROUP_PASSES; p++, ctr += 2) {
-            const int last = p == GROUP_PASSES - 1;
-            if (p == 0) launch_search<P, SETS, true>(a, b, c0, nc, ctr, MODE, sm_count, s);
-            else launch_search<P, SETS, false>(a, b, c0, nc, ctr, MODE, sm_count, s);
-            launch_gclip<P, G, SETS>(a, b, c0, nc, ctr + 1, last, sm_count, s);
+        // counters of a pass: search queue, clip queue, cells listed for the next pass.  The first passes take the
+        // chunk's cells in order (neighbours search together); from pass GLIST on the few left are listed
+        for (int p = 0; p < passes; p++, ctr += 4) {
+            const int last = p == passes - 1;
+            const uint32_t *act = p < GLIST ? nullptr : b.act + (size_t)(p & 1) * b.chunk, *n_act = p < GLIST ? nullptr : ctr - 2;
+            uint32_t* next = p >= GLIST - 1 && !last ? b.act + (size_t)((p + 1) & 1) * b.chunk : nullptr;
+            if (p == 0) launch_search<P, SETS, true>(a, b, c0, nc, ctr, MODE, act, n_act, sm_count, s);
+            else launch_search<P, SETS, false>(a, b, c0, nc, ctr, MODE, act, n_act, sm_count, s);
+            launch_gclip<P, G, SETS>(a, b, c0, nc, ctr + 1, last, act, n_act, next, ctr + 2, sm_count, s);
             n += 2;
         }
     }

@@ -134,6 +134,7 @@ struct vt_handle_s {
     void* g_hdr;
     uint32_t* g_list;
     unsigned char* g_state;
+    uint32_t* g_act;
     uint32_t* g_ctr;
     // scratch for sort / scans
     void* tmp;

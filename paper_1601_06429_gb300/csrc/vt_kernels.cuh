@@ -81,7 +81,7 @@ struct ClipArgs {
 constexpr int GROUP_CAND = 96;
 constexpr int GROUP_NT = 64, GROUP_NP = 40;  // vertex slots and planes of a cell
 constexpr int GROUP_STATE = (GROUP_NT * 20 + GROUP_NP * 21 + 15) / 16 * 16;
-constexpr int GROUP_PASSES = 8;
+constexpr int GROUP_PASSES = 12;
 constexpr uint32_t GROUP_CHUNK = 1u << 21;
 struct GHdr {
     float rlo2, rhi2, B, R2, cap2;            // range of |d|^2 of the pass, start box, squared radius, widest search
@@ -94,6 +94,7 @@ struct GroupBuf {
     GHdr* hdr;
     uint32_t* list;        // [GROUP_CAND] a cell, in order of distance
     unsigned char* state;  // [GROUP_STATE] a cell
+    uint32_t* act;         // [2 * chunk] cells listed for a pass
     uint32_t* ctr;         // [group_counters(N)], zero before the launches
     uint32_t chunk;        // cells of a chunk (a multiple of 32)
 };
@@ -102,7 +103,7 @@ inline uint32_t group_chunk(int64_t N) {
     return n < (int64_t)GROUP_CHUNK ? (uint32_t)n : GROUP_CHUNK;
 }
 inline size_t group_counters(int64_t N) {
-    return 2 * 2 * (size_t)GROUP_PASSES * (size_t)((N + group_chunk(N) - 1) / group_chunk(N));
+    return 2 * 4 * (size_t)GROUP_PASSES * (size_t)((N + group_chunk(N) - 1) / group_chunk(N));
 }
 int launch_clip(const ClipArgs& a, const GroupBuf* gb, int dtype, int precision, int sm_count, cudaStream_t s);
 int launch_clip_exact(const ClipArgs& a, int dtype, int sm_count, cudaStream_t s);
