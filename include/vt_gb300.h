@@ -307,9 +307,9 @@ int vt_grid_density(vt_handle h, int G, int S, void *grid);
  * "average Voronoi densities on a regular grid", read exactly):
  *   grid[v] = sum_i rho_i |V_i intersect voxel v| / |voxel v|,
  * voxel (a, b, c) = [lo + a L/G, lo + (a+1) L/G] per axis (x fastest in grid,
- * device [G][G][G], dtype of pos); periodic boxes wrap.  Each cell is rebuilt
- * from its facet planes and clipped by the walls of every voxel it meets, in
- * FP32 (volumes to about 1e-6 relative).  1 <= G <= 1024.  Allocates, on the
+ * device [G][G][G], dtype of pos); periodic boxes wrap.  Each voxel is cut by
+ * the facet planes of every cell that meets it, in FP32 (volumes to about 1e-6
+ * relative).  1 <= G <= 1024.  Allocates, on the
  * first call (and for a larger G), an FP64 accumulator of G^3 and a retry
  * list; parts that cannot be computed are counted in vt_stats.n_grid_failed.
  * VT_ERR_UNSUPPORTED on a vt_build_batched handle.

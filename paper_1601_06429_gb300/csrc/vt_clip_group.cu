@@ -26,6 +26,7 @@
 #include <cstddef>
 
 #include "vt_clip_impl.cuh"
+#include "vt_grid.cuh"
 
 namespace vt {
 namespace {
@@ -736,6 +737,165 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
     }
 }
 
+// Cut the cells of the groups with `cut` set by the plane that lane `src` of the group holds (pl, from its lane's particle
+// `from`), which removes exactly the vertex slots rem: the plane gets an id, every edge between a removed and a kept vertex
+// becomes a new vertex (w: the new slots).  fail is set where the cell outgrows its capacity or a vertex is
+// ill-conditioned.  The whole warp calls.
+template <int G>
+__device__ __forceinline__ void group_cut(GCell& C, bool& cut, int src, unsigned rem0, unsigned rem1, float4 pl, uint32_t from,
+                                          unsigned& vlo, unsigned& vhi, int& np, int& nseq, int& fail, unsigned& w0,
+                                          unsigned& w1) {
+    const unsigned lane = lane_id();
+    const int r = (int)(lane & (G - 1)), gsh = (int)(lane & ~(unsigned)(G - 1));
+    if (__any_sync(FULL, cut && np == GNP)) {
+        // planes no vertex uses any more are dropped (the start walls keep their ids, the others their order)
+        const bool cp = cut && np == GNP;
+        unsigned use0 = 0u, use1 = 0u;
+#pragma unroll 1
+        for (int s = r; s < GNT; s += G)
+            if (cp && in_set(vlo, vhi, (uint32_t)s)) {
+                uint32_t a, b, c;
+                ids_of(C.V[s].w, a, b, c);
+                const unsigned long long mk = (1ull << a) | (1ull << b) | (1ull << c);
+                use0 |= (unsigned)mk; use1 |= (unsigned)(mk >> 32);
+            }
+        const unsigned long long use = ((unsigned long long)gor<G>(use1) << 32) | gor<G>(use0) | 0x3full;
+#pragma unroll 1
+        for (int p = r; p < GNP; p += G) {
+            const bool mv = cp && ((use >> p) & 1ull);
+            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+            uint32_t qs = 0u;
+            uint8_t qq = 0;
+            if (mv) { q = C.Pl[p]; qs = C.Ps[p]; qq = C.Sq[p]; }
+            __syncwarp();
+            const int d = __popcll(use & ((1ull << p) - 1ull));
+            if (mv) { C.Pl[d] = q; C.Ps[d] = qs; C.Sq[d] = qq; }
+            __syncwarp();
+        }
+#pragma unroll 1
+        for (int s = r; s < GNT; s += G)
+            if (cp && in_set(vlo, vhi, (uint32_t)s)) {
+                uint32_t a, b, c;
+                const uint32_t w = __float_as_uint(C.V[s].w);
+                ids_of(C.V[s].w, a, b, c);
+                C.V[s].w = __uint_as_float((w & ~IDS) | pack_ids(__popcll(use & ((1ull << a) - 1ull)), __popcll(use & ((1ull << b) - 1ull)),
+                                                                  __popcll(use & ((1ull << c) - 1ull))));
+            }
+        if (cp) {
+            np = __popcll(use);
+            if (np == GNP || nseq > 127) { fail = GF_CAP; cut = false; }
+        }
+        __syncwarp();
+    }
+    const int p = np;
+    if (cut) {
+        if (lane == (unsigned)src) {
+            C.Pl[p] = pl;
+            C.Ps[p] = from;
+            C.Sq[p] = (uint8_t)nseq;
+        }
+        np++;
+        nseq++;
+    }
+    // boundary edges: edge k of a removed vertex whose neighbour across it is kept; numbered by chunk of
+    // 32 slots, edge, slot
+    int nB = 0;
+#pragma unroll 1
+    for (int e = 0; e < 2; e++) {
+        const unsigned re = cut ? (e ? rem1 : rem0) : 0u;
+        if (!__any_sync(FULL, re != 0u)) continue;
+        unsigned first = re;
+#pragma unroll
+        for (int q = 0; q < G - 1; q++)
+            if (q < r) first &= first - 1u;
+        unsigned b0 = 0u, b1 = 0u, b2 = 0u;
+        unsigned mm = first;
+#pragma unroll 1
+        while (__any_sync(FULL, mm != 0u)) {
+            if (mm) {
+                const unsigned bit = mm & (0u - mm);
+                const uint32_t ad = C.Ad[e * 32 + __ffs(mm) - 1];
+                if (!in_set(rem0, rem1, ad & 255u)) b0 |= bit;
+                if (!in_set(rem0, rem1, (ad >> 8) & 255u)) b1 |= bit;
+                if (!in_set(rem0, rem1, (ad >> 16) & 255u)) b2 |= bit;
+            }
+#pragma unroll
+            for (int q = 0; q < G; q++) mm &= mm - 1u;
+        }
+        b0 = gor<G>(b0); b1 = gor<G>(b1); b2 = gor<G>(b2);
+        const int n0 = __popc(b0), n1 = __popc(b1), n2 = __popc(b2);
+        mm = first;
+#pragma unroll 1
+        while (__any_sync(FULL, mm != 0u)) {
+            if (mm) {
+                const unsigned bit = mm & (0u - mm);
+                const uint32_t t = (uint32_t)(e * 32 + __ffs(mm) - 1);
+                const uint32_t ad = C.Ad[t], tr = __float_as_uint(C.V[t].w);
+#pragma unroll
+                for (int q = 0; q < 3; q++) {
+                    const unsigned bq = q == 0 ? b0 : q == 1 ? b1 : b2;
+                    if (!(bq & bit)) continue;
+                    const int o = nB + (q > 0 ? n0 : 0) + (q > 1 ? n1 : 0) + __popc(bq & (bit - 1u));
+                    const uint32_t nb = (ad >> (8 * q)) & 63u;
+                    const uint32_t na = C.Ad[nb];
+                    const uint32_t kn = (na & 255u) == t ? 0u : ((na >> 8) & 255u) == t ? 1u : 2u;
+                    const uint32_t x = (tr >> (IDB5 * q)) & IDM5, y = (tr >> (q == 2 ? 0 : IDB5 * (q + 1))) & IDM5;
+                    if (o < GBND) C.bnd[o] = x | (y << 6) | (nb << 12) | (kn << 18);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < G; q++) mm &= mm - 1u;
+        }
+        nB += n0 + n1 + n2;
+    }
+    unsigned long long fr = ~((((unsigned long long)vhi << 32) | vlo) & ~(((unsigned long long)rem1 << 32) | rem0)) &
+                            (GNT == 64 ? ~0ull : (1ull << (GNT & 63)) - 1ull);
+    if (cut && (nB > min(GBND, __popcll(fr)) || nB < 3)) { fail = GF_CAP; cut = false; }
+    if (!cut) nB = 0;
+    __syncwarp();
+    // the i-th boundary edge takes the i-th lowest free slot
+    w0 = w1 = 0u;
+#pragma unroll
+    for (int q = 0; q < G - 1; q++)
+        if (q < r) fr &= fr - 1ull;
+    const int nBmax = __reduce_max_sync(FULL, nB);
+#pragma unroll 1
+    for (int i = r; i < nBmax; i += G) {
+        if (i < nB) {
+            const uint32_t t = (uint32_t)__ffsll((long long)fr) - 1u;
+            const uint32_t rec = C.bnd[i];
+            C.lnk_s[rec & 63u] = (uint8_t)t;
+            C.lnk_e[(rec >> 6) & 63u] = (uint8_t)t;
+            C.bnd[i] = rec | (t << 20);
+            if (t < 32) w0 |= 1u << t; else w1 |= 1u << (t - 32);
+        }
+#pragma unroll
+        for (int q = 0; q < G; q++) fr &= fr - 1ull;
+    }
+    __syncwarp();
+    bool ill = false;
+#pragma unroll 1
+    for (int i = r; i < nBmax; i += G) {
+        if (i < nB) {
+            const uint32_t rec = C.bnd[i];
+            const uint32_t x = rec & 63u, y = (rec >> 6) & 63u, nb = (rec >> 12) & 63u, kn = (rec >> 18) & 3u,
+                           t = rec >> 20;
+            C.Ad[t] = nb | ((uint32_t)C.lnk_s[y] << 8) | ((uint32_t)C.lnk_e[x] << 16);
+            reinterpret_cast<uint8_t*>(&C.Ad[nb])[kn] = (uint8_t)t;
+            float rr;
+            const float4 v = vertex_at(C, x, y, (uint32_t)p, rr);
+            C.V[t] = make_float4(v.x, v.y, v.z, pack_w(v.w, pack_ids(x, y, (uint32_t)p)));
+            if (!(v.w < INFINITY)) ill = true;
+        }
+    }
+    w0 = gor<G>(w0); w1 = gor<G>(w1);
+    if (cut) {
+        vlo = (vlo & ~rem0) | w0;
+        vhi = (vhi & ~rem1) | w1;
+    }
+    if ((__ballot_sync(FULL, ill) >> gsh) & ((1u << G) - 1u)) fail = GF_ILL;
+}
+
 // Clip the cells [c0, c0 + nc) that want a pass by their candidate lists.  last: cells that want another pass are handed
 // over.
 template <typename P, int G, bool SETS>
@@ -966,155 +1126,10 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
                 if (!__any_sync(FULL, cut)) break;
                 const int src = gsh + (cut ? __ffs(cm) - 1 : 0);
                 const unsigned rem0 = __shfl_sync(FULL, olo, src), rem1 = __shfl_sync(FULL, ohi, src);
-                if (__any_sync(FULL, cut && np == GNP)) {
-                    // planes no vertex uses any more are dropped (the start walls keep their ids, the others their order)
-                    const bool cp = cut && np == GNP;
-                    unsigned use0 = 0u, use1 = 0u;
-#pragma unroll 1
-                    for (int s = r; s < GNT; s += G)
-                        if (cp && in_set(vlo, vhi, (uint32_t)s)) {
-                            uint32_t a, b, c;
-                            ids_of(C.V[s].w, a, b, c);
-                            const unsigned long long mk = (1ull << a) | (1ull << b) | (1ull << c);
-                            use0 |= (unsigned)mk; use1 |= (unsigned)(mk >> 32);
-                        }
-                    const unsigned long long use = ((unsigned long long)gor<G>(use1) << 32) | gor<G>(use0) | 0x3full;
-#pragma unroll 1
-                    for (int p = r; p < GNP; p += G) {
-                        const bool mv = cp && ((use >> p) & 1ull);
-                        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-                        uint32_t qs = 0u;
-                        uint8_t qq = 0;
-                        if (mv) { q = C.Pl[p]; qs = C.Ps[p]; qq = C.Sq[p]; }
-                        __syncwarp();
-                        const int d = __popcll(use & ((1ull << p) - 1ull));
-                        if (mv) { C.Pl[d] = q; C.Ps[d] = qs; C.Sq[d] = qq; }
-                        __syncwarp();
-                    }
-#pragma unroll 1
-                    for (int s = r; s < GNT; s += G)
-                        if (cp && in_set(vlo, vhi, (uint32_t)s)) {
-                            uint32_t a, b, c;
-                            const uint32_t w = __float_as_uint(C.V[s].w);
-                            ids_of(C.V[s].w, a, b, c);
-                            C.V[s].w = __uint_as_float((w & ~IDS) | pack_ids(__popcll(use & ((1ull << a) - 1ull)), __popcll(use & ((1ull << b) - 1ull)),
-                                                                              __popcll(use & ((1ull << c) - 1ull))));
-                        }
-                    if (cp) {
-                        np = __popcll(use);
-                        if (np == GNP || nseq > 127) { fail = GF_CAP; cut = false; }
-                    }
-                    __syncwarp();
-                }
-                const int p = np;
-                if (cut) {
-                    if (lane == (unsigned)src) {
-                        C.Pl[p] = make_float4(cdx, cdy, cdz, chh);
-                        C.Ps[p] = cjj;
-                        C.Sq[p] = (uint8_t)nseq;
-                    }
-                    np++;
-                    nseq++;
-                    c_cut += r == 0;
-                    dirty++;
-                }
-                // boundary edges: edge k of a removed vertex whose neighbour across it is kept; numbered by chunk of
-                // 32 slots, edge, slot
-                int nB = 0;
-#pragma unroll 1
-                for (int e = 0; e < 2; e++) {
-                    const unsigned re = cut ? (e ? rem1 : rem0) : 0u;
-                    if (!__any_sync(FULL, re != 0u)) continue;
-                    unsigned first = re;
-#pragma unroll
-                    for (int q = 0; q < G - 1; q++)
-                        if (q < r) first &= first - 1u;
-                    unsigned b0 = 0u, b1 = 0u, b2 = 0u;
-                    unsigned mm = first;
-#pragma unroll 1
-                    while (__any_sync(FULL, mm != 0u)) {
-                        if (mm) {
-                            const unsigned bit = mm & (0u - mm);
-                            const uint32_t ad = C.Ad[e * 32 + __ffs(mm) - 1];
-                            if (!in_set(rem0, rem1, ad & 255u)) b0 |= bit;
-                            if (!in_set(rem0, rem1, (ad >> 8) & 255u)) b1 |= bit;
-                            if (!in_set(rem0, rem1, (ad >> 16) & 255u)) b2 |= bit;
-                        }
-#pragma unroll
-                        for (int q = 0; q < G; q++) mm &= mm - 1u;
-                    }
-                    b0 = gor<G>(b0); b1 = gor<G>(b1); b2 = gor<G>(b2);
-                    const int n0 = __popc(b0), n1 = __popc(b1), n2 = __popc(b2);
-                    mm = first;
-#pragma unroll 1
-                    while (__any_sync(FULL, mm != 0u)) {
-                        if (mm) {
-                            const unsigned bit = mm & (0u - mm);
-                            const uint32_t t = (uint32_t)(e * 32 + __ffs(mm) - 1);
-                            const uint32_t ad = C.Ad[t], tr = __float_as_uint(C.V[t].w);
-#pragma unroll
-                            for (int q = 0; q < 3; q++) {
-                                const unsigned bq = q == 0 ? b0 : q == 1 ? b1 : b2;
-                                if (!(bq & bit)) continue;
-                                const int o = nB + (q > 0 ? n0 : 0) + (q > 1 ? n1 : 0) + __popc(bq & (bit - 1u));
-                                const uint32_t nb = (ad >> (8 * q)) & 63u;
-                                const uint32_t na = C.Ad[nb];
-                                const uint32_t kn = (na & 255u) == t ? 0u : ((na >> 8) & 255u) == t ? 1u : 2u;
-                                const uint32_t x = (tr >> (IDB5 * q)) & IDM5, y = (tr >> (q == 2 ? 0 : IDB5 * (q + 1))) & IDM5;
-                                if (o < GBND) C.bnd[o] = x | (y << 6) | (nb << 12) | (kn << 18);
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < G; q++) mm &= mm - 1u;
-                    }
-                    nB += n0 + n1 + n2;
-                }
-                unsigned long long fr = ~((((unsigned long long)vhi << 32) | vlo) & ~(((unsigned long long)rem1 << 32) | rem0)) &
-                                        (GNT == 64 ? ~0ull : (1ull << (GNT & 63)) - 1ull);
-                if (cut && (nB > min(GBND, __popcll(fr)) || nB < 3)) { fail = GF_CAP; cut = false; }
-                if (!cut) nB = 0;
-                __syncwarp();
-                // the i-th boundary edge takes the i-th lowest free slot
-                unsigned w0 = 0u, w1 = 0u;
-#pragma unroll
-                for (int q = 0; q < G - 1; q++)
-                    if (q < r) fr &= fr - 1ull;
-                const int nBmax = __reduce_max_sync(FULL, nB);
-#pragma unroll 1
-                for (int i = r; i < nBmax; i += G) {
-                    if (i < nB) {
-                        const uint32_t t = (uint32_t)__ffsll((long long)fr) - 1u;
-                        const uint32_t rec = C.bnd[i];
-                        C.lnk_s[rec & 63u] = (uint8_t)t;
-                        C.lnk_e[(rec >> 6) & 63u] = (uint8_t)t;
-                        C.bnd[i] = rec | (t << 20);
-                        if (t < 32) w0 |= 1u << t; else w1 |= 1u << (t - 32);
-                    }
-#pragma unroll
-                    for (int q = 0; q < G; q++) fr &= fr - 1ull;
-                }
-                __syncwarp();
-                bool ill = false;
-#pragma unroll 1
-                for (int i = r; i < nBmax; i += G) {
-                    if (i < nB) {
-                        const uint32_t rec = C.bnd[i];
-                        const uint32_t x = rec & 63u, y = (rec >> 6) & 63u, nb = (rec >> 12) & 63u, kn = (rec >> 18) & 3u,
-                                       t = rec >> 20;
-                        C.Ad[t] = nb | ((uint32_t)C.lnk_s[y] << 8) | ((uint32_t)C.lnk_e[x] << 16);
-                        reinterpret_cast<uint8_t*>(&C.Ad[nb])[kn] = (uint8_t)t;
-                        float rr;
-                        const float4 v = vertex_at(C, x, y, (uint32_t)p, rr);
-                        C.V[t] = make_float4(v.x, v.y, v.z, pack_w(v.w, pack_ids(x, y, (uint32_t)p)));
-                        if (!(v.w < INFINITY)) ill = true;
-                    }
-                }
-                w0 = gor<G>(w0); w1 = gor<G>(w1);
-                if (cut) {
-                    vlo = (vlo & ~rem0) | w0;
-                    vhi = (vhi & ~rem1) | w1;
-                }
-                if (gballot(ill)) fail = GF_ILL;
+                unsigned w0, w1;
+                c_cut += cut && r == 0;
+                dirty += cut;
+                group_cut<G>(C, cut, src, rem0, rem1, make_float4(cdx, cdy, cdz, chh), cjj, vlo, vhi, np, nseq, fail, w0, w1);
                 __syncwarp();
                 // the later planes against the new vertices
                 olo &= ~rem0; ohi &= ~rem1;
@@ -1552,6 +1567,307 @@ int launch_group(const ClipArgs& a, const GroupBuf& b, int sm_count, cudaStream_
     }
     return n;
 }
+// ------------------------------------------------------------------ volume-averaged grid: (cell, voxel) pairs
+// The part of a voxel inside a cell is the voxel cut by the cell's facet planes, and most pairs need no cutting: the
+// voxel lies outside one plane (no part), or inside all of them (all of it); a cell whose ball lies in one voxel gives it
+// its whole volume.  A warp takes 32 cells at a time, its lanes one pair each of all the voxels that the cells' balls
+// meet.  The pairs that some plane crosses wait in queues (of about the same number of crossing planes) until there are
+// enough, and are cut by the crossing planes alone, G lanes a pair as in k_group_clip, starting from the voxel's box (cut
+// down to the ball's).  Sides are plain FP32 signs: a wrong sign within rounding of a plane moves a rounding-sized sliver.
+// Cells whose balls meet more than GV_BIG voxels are listed and a second launch spreads each over all warps.
+// Bound by instruction issue, as k_group_clip.  131,072 clustered particles on 32^3 voxels: 4.7 ms; 297 ms with one thread
+// walking all voxels of a cell and clipping a copy of it by each voxel's walls; 13 ms with one thread a pair (5 of 32 lanes
+// active, and the lanes' polytopes in local memory).
+constexpr int GV_BIG = 512;
+constexpr int GV_CLASSES = 4;
+
+struct GridWarp {
+    int pref[33];
+    int a0[3][32], n[3][32];  // first voxel and number of voxels per axis (unwrapped)
+    int4 q[GV_CLASSES][64];   // pairs to cut, by class
+};
+
+template <typename P, bool BIG>
+__global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ GridArgs A) {
+    constexpr int G = 4, W = 32 / G;
+    extern __shared__ __align__(16) unsigned char gsmem[];
+    GCell* const cells = reinterpret_cast<GCell*>(gsmem);
+    GridWarp& S = *reinterpret_cast<GridWarp*>(cells + W);
+    const unsigned lane = lane_id(), lt = lanemask_lt();
+    const int r = (int)(lane & (G - 1)), gsh = (int)(lane & ~(unsigned)(G - 1));
+    constexpr unsigned GM = (1u << G) - 1u;
+    GCell& C = cells[gsh / G];
+    const P* const spos = (const P*)A.spos;
+    const double vox = A.h[0] * A.h[1] * A.h[2];
+    const unsigned n_big = BIG ? *((volatile unsigned*)A.n_big) : 0u;
+    auto gballot = [&](bool p) -> unsigned { return (__ballot_sync(FULL, p) >> gsh) & GM; };
+    auto gsum = [&](float v) -> float {
+#pragma unroll
+        for (int o = G / 2; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+        return v;
+    };
+    int nq[GV_CLASSES];
+#pragma unroll
+    for (int c = 0; c < GV_CLASSES; c++) nq[c] = 0;
+
+    unsigned e = 0, b = 0;
+    int64_t total = 0, t1 = 0;
+    bool more = true;
+    for (;;) {
+        // ---------------------------------------------------------------- 32 pairs to look at
+        if (t1 >= total && more) {
+            total = 0;
+            if (BIG) {
+                // one listed cell over all warps
+                if (e >= n_big) more = false;
+                else {
+                    const uint32_t k = A.big[e];
+                    const P pi = spos[k];
+                    const double xi[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
+                    int a0[3], n[3];
+                    total = ball_voxels(A, xi, A.rad[k] * (1.f + 4e-6f), a0, n);
+                    if (lane < 3) {
+                        S.a0[lane][0] = lane == 0 ? a0[0] : lane == 1 ? a0[1] : a0[2];
+                        S.n[lane][0] = lane == 0 ? n[0] : lane == 1 ? n[1] : n[2];
+                    }
+                    b = k;
+                    e++;
+                    t1 = (int64_t)blockIdx.x * 32;
+                }
+            } else {
+                if (lane == 0) b = atomicAdd(A.queue, 32u);
+                b = __shfl_sync(FULL, b, 0);
+                if ((int64_t)b >= A.N) more = false;
+                else {
+                    const int64_t k = (int64_t)b + lane;
+                    int m = 0;
+                    if (k < A.N && A.rad[k] > 0.f) {
+                        const P pi = spos[k];
+                        const double xi[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
+                        int a0[3], n[3];
+                        const int64_t mm = ball_voxels(A, xi, A.rad[k] * (1.f + 4e-6f), a0, n);
+                        if (mm == 1) {
+                            int64_t v[3];
+                            for (int c = 0; c < 3; c++) {
+                                const int q = a0[c] % A.G;
+                                v[c] = q < 0 ? q + A.G : q;
+                            }
+                            atomicAdd(&A.acc[(v[2] * A.G + v[1]) * A.G + v[0]], A.dens[k] * A.cell[k].vol);
+                        } else if (mm > GV_BIG) {
+                            A.big[atomicAdd(A.n_big, 1u)] = (uint32_t)k;
+                        } else {
+                            m = (int)mm;
+                            for (int c = 0; c < 3; c++) { S.a0[c][lane] = a0[c]; S.n[c][lane] = n[c]; }
+                        }
+                    }
+                    int x = m;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(FULL, x, o);
+                        if ((int)lane >= o) x += y;
+                    }
+                    S.pref[lane + 1] = x;
+                    if (lane == 0) S.pref[0] = 0;
+                    total = __shfl_sync(FULL, x, 31);
+                    t1 = 0;
+                }
+            }
+            __syncwarp();
+        }
+        if (t1 < total) {
+            const int64_t t = t1 + lane;
+            int cross = -1;
+            int4 ent = make_int4(0, 0, 0, 0);
+            if (t < total) {
+                int c = 0, i = (int)t;
+                if (!BIG) {
+                    // the cell of pair t: the last with pref <= t
+#pragma unroll
+                    for (int o = 16; o; o >>= 1)
+                        if (S.pref[c + o] <= (int)t) c += o;
+                    i -= S.pref[c];
+                }
+                const int n0 = S.n[0][c], n1 = S.n[1][c];
+                const int ia[3] = {S.a0[0][c] + i % n0, S.a0[1][c] + (i / n0) % n1, S.a0[2][c] + i / (n0 * n1)};
+                const uint32_t k = b + (uint32_t)c;
+                const P pi = spos[k];
+                const double xi[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
+                float lo[3], hi[3];
+                const int64_t vi = voxel_box(A, xi, A.rad[k] * (1.f + 4e-6f), ia, lo, hi);
+                cross = side_of_box(A, A.face_start[k], A.face_count[k], lo, hi);
+                if (cross == 0) atomicAdd(&A.acc[vi], A.dens[k] * vox);
+                ent = make_int4((int)k, ia[0], ia[1], ia[2]);
+            }
+            const int cls = cross <= 0 ? -1 : cross <= 2 ? 0 : cross <= 5 ? 1 : cross <= 10 ? 2 : 3;
+#pragma unroll
+            for (int c = 0; c < GV_CLASSES; c++) {
+                const unsigned cm = __ballot_sync(FULL, cls == c);
+                if (cls == c) S.q[c][nq[c] + __popc(cm & lt)] = ent;
+                nq[c] += __popc(cm);
+            }
+            t1 += BIG ? (int64_t)gridDim.x * 32 : 32;
+            __syncwarp();
+        }
+        // ---------------------------------------------------------------- eight pairs of a class, while one is full
+        bool idle = true;
+#pragma unroll 1
+        for (;;) {
+            int cl = -1, m = 0;
+#pragma unroll
+            for (int c = 0; c < GV_CLASSES; c++)
+                if (nq[c] >= 32 || (!more && t1 >= total && nq[c] > 0)) { cl = c; m = nq[c]; }
+            if (cl < 0) break;
+            idle = false;
+            const int take = m < W ? m : W;
+            const bool has = gsh / G < take;
+            const int4 ent = S.q[cl][has ? m - take + gsh / G : 0];
+#pragma unroll
+            for (int c = 0; c < GV_CLASSES; c++)
+                if (c == cl) nq[c] -= take;
+            const uint32_t k = (uint32_t)ent.x, st = A.face_start[k];
+            const int cnt = has ? (int)A.face_count[k] : 0;
+            float lo[3], hi[3];
+            int64_t vi;
+            {
+                const P pi = spos[k];
+                const double xi[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
+                const int ia[3] = {ent.y, ent.z, ent.w};
+                vi = voxel_box(A, xi, A.rad[k] * (1.f + 4e-6f), ia, lo, hi);
+            }
+            // start: the box (walls and corners as in k_group_clip)
+            __syncwarp();
+#pragma unroll 1
+            for (int w = r; w < 6; w += G) {
+                const float sg = (w & 1) ? -1.f : 1.f;
+                const float h = w == 0 ? hi[0] : w == 1 ? -lo[0] : w == 2 ? hi[1] : w == 3 ? -lo[1] : w == 4 ? hi[2] : -lo[2];
+                C.Pl[w] = make_float4(w < 2 ? sg : 0.f, (w >> 1) == 1 ? sg : 0.f, w > 3 ? sg : 0.f, h);
+                C.Ps[w] = 0u;
+                C.Sq[w] = (uint8_t)w;
+            }
+#pragma unroll 1
+            for (int q = r; q < 8; q += G) {
+                const bool even = (__popc((unsigned)q) & 1) == 0;
+                const uint32_t X = (q & 1) ? 1 : 0, Y = (q & 2) ? 3 : 2, Z = (q & 4) ? 5 : 4;
+                C.V[q] = make_float4((q & 1) ? lo[0] : hi[0], (q & 2) ? lo[1] : hi[1], (q & 4) ? lo[2] : hi[2],
+                                     pack_w(0.f, pack_ids(X, even ? Y : Z, even ? Z : Y)));
+                const uint32_t fx = (uint32_t)q ^ 1u, fy = (uint32_t)q ^ 2u, fz = (uint32_t)q ^ 4u;
+                C.Ad[q] = even ? (fz | (fx << 8) | (fy << 16)) : (fy | (fx << 8) | (fz << 16));
+            }
+            unsigned vlo = has ? 0xffu : 0u, vhi = 0u;
+            int np = 6, nseq = 6, fail = 0;
+            bool empty = !has;
+            __syncwarp();
+            // the planes in batches of G, one per lane, as in k_group_clip
+#pragma unroll 1
+            for (int base = 0;; base += G) {
+                const bool open = !fail && !empty && base < cnt;
+                if (!__any_sync(FULL, open)) break;
+                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+                bool on = open && base + r < cnt;
+                if (on) {
+                    f = *reinterpret_cast<const float4*>(&A.faces[st + base + r]);
+                    f.w = 0.5f * __fmaf_rn(f.z, f.z, __fmaf_rn(f.y, f.y, f.x * f.x));
+                    on = fmaxf(f.x * lo[0], f.x * hi[0]) + fmaxf(f.y * lo[1], f.y * hi[1]) + fmaxf(f.z * lo[2], f.z * hi[2]) > f.w;
+                }
+                if (!__any_sync(FULL, on)) continue;
+                unsigned olo = 0u, ohi = 0u;
+                const int hw = open ? (vhi ? 64 - __clz(vhi) : 32 - __clz(vlo)) : 0;
+                const int hmax = __reduce_max_sync(FULL, hw);
+#pragma unroll 1
+                for (int s0 = 0; s0 < hmax; s0 += 4) {
+                    unsigned o4 = 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const float4 v = C.V[s0 + q];
+                        if (f_fma<float>(f.x, v.x, f_fma<float>(f.y, v.y, f_fma<float>(f.z, v.z, -f.w))) > 0.f) o4 |= 1u << q;
+                    }
+                    if (s0 < 32) olo |= o4 << s0;
+                    else ohi |= o4 << (s0 - 32);
+                }
+                olo = on ? olo & vlo : 0u;
+                ohi = on ? ohi & vhi : 0u;
+#pragma unroll 1
+                for (;;) {
+                    const unsigned cm = gballot((olo | ohi) != 0u);
+                    bool cut = open && !fail && !empty && cm != 0u;
+                    if (!__any_sync(FULL, cut)) break;
+                    const int src = gsh + (cut ? __ffs(cm) - 1 : 0);
+                    const unsigned rem0 = __shfl_sync(FULL, olo, src), rem1 = __shfl_sync(FULL, ohi, src);
+                    if (cut && rem0 == vlo && rem1 == vhi) {  // nothing is left
+                        empty = true;
+                        cut = false;
+                    }
+                    unsigned w0, w1;
+                    group_cut<G>(C, cut, src, rem0, rem1, f, 0u, vlo, vhi, np, nseq, fail, w0, w1);
+                    __syncwarp();
+                    olo &= ~rem0; ohi &= ~rem1;
+                    if ((int)lane <= src || !cut) olo = ohi = 0u;
+                    const bool later = on && cut && (int)lane > src;
+                    unsigned m0 = cut ? w0 : 0u, m1 = cut ? w1 : 0u;
+#pragma unroll 1
+                    while (__any_sync(FULL, (m0 | m1) != 0u)) {
+                        const int s = m0 ? __ffs(m0) - 1 : m1 ? 31 + __ffs(m1) : 0;
+                        if (m0) m0 &= m0 - 1u; else m1 &= m1 - 1u;
+                        const float4 v = C.V[s];
+                        if (later && f_fma<float>(f.x, v.x, f_fma<float>(f.y, v.y, f_fma<float>(f.z, v.z, -f.w))) > 0.f) {
+                            if (s < 32) olo |= 1u << s; else ohi |= 1u << (s - 32);
+                        }
+                    }
+                }
+            }
+            // the volume from the edges: the edge a->b of a vertex leads to the vertex across it and bounds the face of
+            // plane b, so a face's area is the sum of n.(w x w') / 2 over its edges, w relative to the mean vertex, and
+            // the volume a third of offset times area
+            const bool on = has && !fail && !empty;
+            float sx = 0.f, sy = 0.f, sz = 0.f;
+#pragma unroll 1
+            for (int s = r; s < GNT; s += G)
+                if (on && in_set(vlo, vhi, (uint32_t)s)) {
+                    const float4 v = C.V[s];
+                    sx += v.x; sy += v.y; sz += v.z;
+                }
+            const float im = 1.f / (float)max(1, __popc(vlo) + __popc(vhi));
+            const float mx = gsum(sx) * im, my = gsum(sy) * im, mz = gsum(sz) * im;
+            float vol = 0.f;
+#pragma unroll 1
+            for (int s = r; s < GNT; s += G)
+                if (on && in_set(vlo, vhi, (uint32_t)s)) {
+                    const float4 v = C.V[s];
+                    const float ax = v.x - mx, ay = v.y - my, az = v.z - mz;
+                    uint32_t id[3];
+                    ids_of(v.w, id[0], id[1], id[2]);
+                    const uint32_t ad = C.Ad[s];
+#pragma unroll
+                    for (int q = 0; q < 3; q++) {
+                        const float4 o = C.V[(ad >> (8 * q)) & 63u];
+                        const uint32_t y = id[q == 2 ? 0 : q + 1];
+                        const float4 p = C.Pl[y];
+                        const float bx = o.x - mx, by = o.y - my, bz = o.z - mz;
+                        const float off = p.w - (p.x * mx + p.y * my + p.z * mz);
+                        const float cr = p.x * (ay * bz - az * by) + p.y * (az * bx - ax * bz) + p.z * (ax * by - ay * bx);
+                        vol += y < 6 ? off * cr : off * cr / (2.f * p.w);
+                    }
+                }
+            vol = gsum(vol) * (float)(1.0 / 6.0);
+            if (r == 0 && has) {
+                // a sliver's FP32 volume may come out slightly below zero; anything beyond 1e-5 of the box is a failure
+                if (fail || (on && vol < -1e-5f * (hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])))
+                    push_retry(A, (int64_t)k, ent.y, ent.z, ent.w);
+                else if (on && vol > 0.f) atomicAdd(&A.acc[vi], A.dens[k] * (double)vol);
+            }
+            __syncwarp();
+        }
+        if (!more && t1 >= total && idle) break;
+    }
+}
+
+template <typename P, bool BIG>
+void launch_voxels(const GridArgs& a, int sm_count, cudaStream_t s) {
+    static int per_sm_dev[64] = {0};
+    const size_t smem = 8 * sizeof(GCell) + sizeof(GridWarp);
+    const int per_sm = blocks_per_sm(k_group_voxels<P, BIG>, 32, smem, per_sm_dev);
+    k_group_voxels<P, BIG><<<(unsigned)(sm_count * per_sm), 32, smem, s>>>(a);
+}
 }  // namespace
 
 int launch_clip_group(const ClipArgs& a, const GroupBuf& b, int dtype, int lanes, int sm_count, cudaStream_t s) {
@@ -1561,6 +1877,17 @@ int launch_clip_group(const ClipArgs& a, const GroupBuf& b, int dtype, int lanes
     }
     if (lanes == 4) return a.sset ? launch_group<dpt4, 4, true>(a, b, sm_count, s) : launch_group<dpt4, 4, false>(a, b, sm_count, s);
     return a.sset ? launch_group<dpt4, 8, true>(a, b, sm_count, s) : launch_group<dpt4, 8, false>(a, b, sm_count, s);
+}
+
+int launch_grid_pairs(const GridArgs& a, int dtype, int sm_count, cudaStream_t s) {
+    if (dtype == VT_F32) {
+        launch_voxels<float4, false>(a, sm_count, s);
+        launch_voxels<float4, true>(a, sm_count, s);
+    } else {
+        launch_voxels<dpt4, false>(a, sm_count, s);
+        launch_voxels<dpt4, true>(a, sm_count, s);
+    }
+    return 2;
 }
 
 }  // namespace vt

@@ -20,6 +20,7 @@
 #include <climits>
 
 #include "vt_clip_impl.cuh"
+#include "vt_grid.cuh"
 
 namespace vt {
 namespace {
@@ -939,23 +940,6 @@ __device__ int cut_plain(CL& C, float nx, float ny, float nz, float h, float nrm
     return f ? -f : 0;
 }
 
-struct GridArgs {
-    const void* spos;
-    int64_t N;
-    Geometry geo;
-    const Face* faces;
-    const uint32_t* face_start;
-    const uint16_t* face_count;
-    const double* dens;  // sorted order
-    int G;
-    double h[3];         // voxel side L / G
-    double* acc;         // [G^3] sum of rho |cell & voxel|
-    int4* retry;         // (cell, voxel x, y, z unwrapped; x = INT_MIN: every voxel) for the larger cell type
-    unsigned retry_cap;
-    unsigned* n_retry;
-    unsigned* n_fail;
-};
-
 // The cell of sorted particle k from its facet planes (start: a cube of half-side lmin/4, which holds every cell
 // the build accepted, or the box walls).  Returns 0 or a failure code.
 template <typename P, class CL>
@@ -1034,70 +1018,26 @@ __device__ int voxel_part_retry(const CL& C, CL& D, const GridArgs& A, const dou
     return e;
 }
 
-// a part that cannot be computed: counted in total and by reason (counters[4 + code])
-__device__ __forceinline__ void grid_fail(const GridArgs& A, int code) {
-    atomicAdd(A.n_fail, 1u);
-    atomicAdd(A.n_fail + 3 + (code > 0 && code < 12 ? code : 0), 1u);
-}
-
-__device__ __forceinline__ void push_retry(const GridArgs& A, int64_t k, int ax, int ay, int az) {
-    const unsigned slot = atomicAdd(A.n_retry, 1u);
-    if (slot < A.retry_cap) A.retry[slot] = make_int4((int)k, ax, ay, az);
-    else grid_fail(A, 11);
-}
-
-// One thread per cell (RETRY = false) or per retry entry (RETRY = true, the larger cell type): rho times the
-// volume of the cell inside each voxel its box meets is added to that voxel.  A pair the small cell type
-// cannot hold goes to the retry list, so that no voxel receives a part twice.
-template <typename P, class CL, bool RETRY>
+// The retry pass: one thread per entry, the cell rebuilt in the larger cell type and cut by the voxel's walls.
+template <typename P, class CL>
 __global__ void __launch_bounds__(128) k_grid_volume(GridArgs A) {
-    const int64_t n = RETRY ? (int64_t)min(*((volatile unsigned*)A.n_retry), A.retry_cap) : A.N;
+    const int64_t n = (int64_t)min(*((volatile unsigned*)A.n_retry), A.retry_cap);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        int4 ent = make_int4(0, INT_MIN, 0, 0);
-        if (RETRY) ent = A.retry[e];
-        const int64_t k = RETRY ? (int64_t)ent.x : e;
+        const int4 ent = A.retry[e];
+        const int64_t k = (int64_t)ent.x;
         const P pi = ((const P*)A.spos)[k];
         CL C, D;
-        int f = grid_cell<P, CL>(C, A, k, pi);
+        const int f = grid_cell<P, CL>(C, A, k, pi);
         if (f) {
-            if (!RETRY) push_retry(A, k, INT_MIN, 0, 0);
-            else grid_fail(A, f);
+            grid_fail(A, f);
             continue;
         }
         const double xi[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
-        const double rho = A.dens[k];
-        if (RETRY && ent.y != INT_MIN) {
-            float vol;
-            int64_t vi;
-            const int e2 = voxel_part_retry(C, D, A, xi, ent.y, ent.z, ent.w, &vol, &vi);
-            if (e2) grid_fail(A, e2);
-            else if (vol > 0.f) atomicAdd(&A.acc[vi], rho * (double)vol);
-            continue;
-        }
-        const Geometry& g = A.geo;
-        int64_t a0[3], a1[3];
-        for (int c = 0; c < 3; c++) {
-            a0[c] = (int64_t)floor((xi[c] + (double)C.bmin[c] - g.lo[c]) / A.h[c]) - 1;
-            a1[c] = (int64_t)floor((xi[c] + (double)C.bmax[c] - g.lo[c]) / A.h[c]) + 1;
-            if (!g.periodic) {
-                a0[c] = a0[c] < 0 ? 0 : a0[c];
-                a1[c] = a1[c] > A.G - 1 ? A.G - 1 : a1[c];
-            }
-        }
-        for (int64_t az = a0[2]; az <= a1[2]; az++)
-            for (int64_t ay = a0[1]; ay <= a1[1]; ay++)
-                for (int64_t ax = a0[0]; ax <= a1[0]; ax++) {
-                    float vol;
-                    int64_t vi;
-                    const int e2 = RETRY ? voxel_part_retry(C, D, A, xi, ax, ay, az, &vol, &vi)
-                                         : voxel_part(C, D, A, xi, ax, ay, az, 0.0, &vol, &vi);
-                    if (e2) {
-                        if (!RETRY) push_retry(A, k, (int)ax, (int)ay, (int)az);
-                        else grid_fail(A, e2);
-                    } else if (vol > 0.f) {
-                        atomicAdd(&A.acc[vi], rho * (double)vol);
-                    }
-                }
+        float vol;
+        int64_t vi;
+        const int e2 = voxel_part_retry(C, D, A, xi, ent.y, ent.z, ent.w, &vol, &vi);
+        if (e2) grid_fail(A, e2);
+        else if (vol > 0.f) atomicAdd(&A.acc[vi], A.dens[k] * (double)vol);
     }
 }
 
@@ -1239,8 +1179,8 @@ __global__ void k_grid_finish(const double* __restrict__ acc, int64_t n, double 
 }  // namespace
 
 int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
-                       const uint32_t* face_start, const uint16_t* face_count, const double* dens_sorted, int G,
-                       double* acc, int4* retry, unsigned retry_cap, unsigned* counters, void* out, int sm_count,
+                       const uint32_t* face_start, const uint16_t* face_count, const double* dens_sorted, const float* rad,
+                       const CellOut* cell, uint32_t* big, int G, double* acc, int4* retry, unsigned retry_cap, unsigned* counters, void* out, int sm_count,
                        cudaStream_t s) {
     GridArgs a;
     a.spos = spos; a.N = N; a.geo = g; a.faces = faces; a.face_start = face_start; a.face_count = face_count;
@@ -1250,20 +1190,20 @@ int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g
     const int64_t n = (int64_t)G * G * G;
     cudaMemsetAsync(acc, 0, n * sizeof(double), s);
     cudaMemsetAsync(counters, 0, 16 * sizeof(unsigned), s);
-    const unsigned nb = (unsigned)((N + 127) / 128);
+    a.rad = rad; a.cell = cell; a.big = big;
+    a.n_big = counters + 2; a.queue = counters + 3;
+    launch_grid_pairs(a, dtype, sm_count, s);
     const unsigned rb = (unsigned)(sm_count * 4);
     if (dtype == VT_F32) {
-        k_grid_volume<float4, TCell, false><<<nb, 128, 0, s>>>(a);
-        k_grid_volume<float4, TCellBig, true><<<rb, 128, 0, s>>>(a);
+        k_grid_volume<float4, TCellBig><<<rb, 128, 0, s>>>(a);
     } else {
-        k_grid_volume<dpt4, TCell, false><<<nb, 128, 0, s>>>(a);
-        k_grid_volume<dpt4, TCellBig, true><<<rb, 128, 0, s>>>(a);
+        k_grid_volume<dpt4, TCellBig><<<rb, 128, 0, s>>>(a);
     }
     const double inv = 1.0 / (a.h[0] * a.h[1] * a.h[2]);
     const unsigned gb = (unsigned)((n + 255) / 256);
     if (dtype == VT_F32) k_grid_finish<float><<<gb, 256, 0, s>>>(acc, n, inv, (float*)out);
     else k_grid_finish<double><<<gb, 256, 0, s>>>(acc, n, inv, (double*)out);
-    return 3;
+    return 4;
 }
 
 int launch_cvt_weighted(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
