@@ -823,7 +823,7 @@ int vt_backward_weighted(vt_handle h, const void* w, void* dE_dpos) {
     int rc = ensure_retry(h);
     if (rc) return rc;
     h->n_launches += launch_cvt_weighted(h->spos, h->dtype, h->N, h->geo, h->faces, h->face_start, h->face_count,
-                                         h->cell, h->perm, w, dE_dpos, h->gretry, GRID_RETRY_CAP, h->gcnt, h->sm_count,
+                                         h->cell, h->rad, h->perm, w, dE_dpos, h->gretry, GRID_RETRY_CAP, h->gcnt, h->sm_count,
                                          h->stream);
     return cuda_rc(cudaGetLastError());
 }

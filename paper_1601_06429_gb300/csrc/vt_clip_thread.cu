@@ -1066,6 +1066,7 @@ struct CvtArgs {
     const uint32_t* face_start;
     const uint16_t* face_count;
     const CellOut* cell;
+    const float* rad;
     const uint32_t* perm;
     const void* w;        // weights, input order, dtype of pos
     int dtype;
@@ -1076,27 +1077,174 @@ struct CvtArgs {
     unsigned* n_fail;
 };
 
-// dE_w/dx_k = 2 w_k V_k (x_k - z_k) + sum over facets (w_k - w_j) / |d| integral_f |y - x_k|^2 (y - x_k) dA, one
-// thread per cell (RETRY: per listed cell, larger cell type); the facet integral over the facet polygon of the cell
-// rebuilt from its facet planes, vertices ordered by angle in the facet plane and fanned.
-template <typename P, class CL, bool RETRY>
+// dE_w/dx_k = 2 w_k V_k (x_k - z_k) + sum over facets (w_k - w_j) / |d| integral_f |y - x_k|^2 (y - x_k) dA.
+
+// A convex polygon in a plane's own coordinates, cut by lines a s + b t <= c
+constexpr int PGON = 24;
+struct Polygon {
+    float2 v[2][PGON];  // the vertices in order, in the buffer `in`
+    int n, in;
+};
+// false when the polygon outgrows its buffer; an empty polygon has n = 0
+__device__ __forceinline__ bool cut_polygon(Polygon& G, float a, float b, float c) {
+    const float2* const v = G.v[G.in];
+    bool out = false;
+    for (int k = 0; k < G.n; k++) out = out || a * v[k].x + b * v[k].y > c;
+    if (!out) return true;
+    float2* const w = G.v[G.in ^ 1];
+    int m = 0;
+    float2 p = v[G.n - 1];
+    float dp = a * p.x + b * p.y - c;
+    for (int k = 0; k < G.n; k++) {
+        const float2 q = v[k];
+        const float dq = a * q.x + b * q.y - c;
+        if ((dp > 0.f) != (dq > 0.f)) {
+            if (m == PGON) return false;
+            const float f = dp / (dp - dq);
+            w[m++] = make_float2(p.x + f * (q.x - p.x), p.y + f * (q.y - p.y));
+        }
+        if (!(dq > 0.f)) {
+            if (m == PGON) return false;
+            w[m++] = q;
+        }
+        p = q;
+        dp = dq;
+    }
+    G.n = m;
+    G.in ^= 1;
+    return true;
+}
+
+// Eight lanes per cell, a facet per lane and turn: the facet is a square in its plane, around the foot of the site and as
+// wide as the cell's ball, cut by the cell's other planes (nearest first) and by the walls of a bounded box, each a line
+// in the plane; nothing but the polygon is held, and no cell is rebuilt.  With y = o + s u + t w on the facet (o the foot,
+// u, w the plane's basis) the integrand is a cubic in s and t, which the degree-3 rule takes exactly on the fan of the
+// polygon.  Bound by the divergence of the cuts (about 14 planes a facet, of which 5 cut; 9 of 32 lanes active).  131,072
+// clustered particles: 1.2 ms; 5.4 ms with one thread rebuilding a cell, 3.3 of it retries of a few large cells.
+constexpr int CVT_LANES = 8;
+template <typename P>
+__global__ void __launch_bounds__(128) k_cvt_facets(CvtArgs A) {
+    const unsigned lane = lane_id();
+    const int r = (int)(lane % CVT_LANES);
+    const int64_t per = (int64_t)blockDim.x / CVT_LANES;
+    const int64_t k0 = (int64_t)blockIdx.x * per + threadIdx.x / CVT_LANES;
+    const bool in = k0 < A.N;
+    const int64_t k = in ? k0 : 0;
+    const P pi = ((const P*)A.spos)[k];
+    const uint32_t st = A.face_start[k], ik = A.perm[k];
+    const int cnt = in ? (int)A.face_count[k] : 0;
+    const double wk = A.dtype == VT_F32 ? (double)((const float*)A.w)[ik] : ((const double*)A.w)[ik];
+    const float D = A.rad[k] * 1.01f;
+    double gx = 0.0, gy = 0.0, gz = 0.0;
+    bool fail = false;
+    Polygon G;
+    for (int q0 = 0; __any_sync(0xffffffffu, q0 < cnt); q0 += CVT_LANES) {
+        const int q = q0 + r;
+        const bool on = q < cnt && !fail;
+        float4 f = make_float4(1.f, 0.f, 0.f, 0.f);
+        if (on) f = *reinterpret_cast<const float4*>(&A.faces[st + q]);
+        const float in1 = 1.f / sqrtf(__fmaf_rn(f.z, f.z, __fmaf_rn(f.y, f.y, f.x * f.x)));
+        const float nx = f.x * in1, ny = f.y * in1, nz = f.z * in1;
+        const float o[3] = {0.5f * f.x, 0.5f * f.y, 0.5f * f.z};
+        float u[3], w[3];
+        if (fabsf(nx) < 0.9f) { u[0] = 0.f; u[1] = nz; u[2] = -ny; }
+        else { u[0] = -nz; u[1] = 0.f; u[2] = nx; }
+        const float iu = 1.f / sqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+        u[0] *= iu; u[1] *= iu; u[2] *= iu;
+        w[0] = ny * u[2] - nz * u[1]; w[1] = nz * u[0] - nx * u[2]; w[2] = nx * u[1] - ny * u[0];
+        G.n = on ? 4 : 0;
+        G.in = 0;
+        G.v[0][0] = make_float2(-D, -D); G.v[0][1] = make_float2(D, -D);
+        G.v[0][2] = make_float2(D, D); G.v[0][3] = make_float2(-D, D);
+        for (int q2 = 0; __any_sync(0xffffffffu, q2 < cnt); q2++) {
+            if (on && q2 < cnt && q2 != q && G.n) {
+                const float4 m = *reinterpret_cast<const float4*>(&A.faces[st + q2]);
+                const float h = 0.5f * __fmaf_rn(m.z, m.z, __fmaf_rn(m.y, m.y, m.x * m.x));
+                if (!cut_polygon(G, m.x * u[0] + m.y * u[1] + m.z * u[2], m.x * w[0] + m.y * w[1] + m.z * w[2],
+                                 h - (m.x * o[0] + m.y * o[1] + m.z * o[2])))
+                    fail = true;
+            }
+            __syncwarp();
+        }
+        if (!A.geo.periodic && on)
+            for (int c = 0; c < 6 && G.n; c++) {
+                const int a = c >> 1;
+                const double xi = a == 0 ? (double)pi.x : a == 1 ? (double)pi.y : (double)pi.z;
+                const float sg = (c & 1) ? -1.f : 1.f;
+                const float h = (c & 1) ? (float)(xi - A.geo.lo[a]) : (float)(A.geo.hi[a] - xi);
+                const float ua = a == 0 ? u[0] : a == 1 ? u[1] : u[2], wa = a == 0 ? w[0] : a == 1 ? w[1] : w[2],
+                            oa = a == 0 ? o[0] : a == 1 ? o[1] : o[2];
+                if (!cut_polygon(G, sg * ua, sg * wa, h - sg * oa)) fail = true;
+            }
+        __syncwarp();
+        if (on && G.n >= 3 && !fail) {
+            // integrals over the facet of rho^2, rho^2 s and rho^2 t, rho^2 = |o|^2 + s^2 + t^2 (the rule of Strang and Fix)
+            const float2* const v = G.v[G.in];
+            const float oo = o[0] * o[0] + o[1] * o[1] + o[2] * o[2];
+            double m0 = 0.0, ms = 0.0, mt = 0.0;
+            for (int e = 1; e + 1 < G.n; e++) {
+                const float2 a = v[0], b = v[e], c = v[e + 1];
+                const float at = 0.5f * ((b.x - a.x) * (c.y - a.y) - (c.x - a.x) * (b.y - a.y));
+                float i0 = 0.f, is = 0.f, it = 0.f;
+#pragma unroll
+                for (int g = 0; g < 4; g++) {
+                    const float wa = g == 0 ? 1.f / 3.f : g == 1 ? 0.6f : 0.2f, wb = g == 0 ? 1.f / 3.f : g == 2 ? 0.6f : 0.2f,
+                                wc = g == 0 ? 1.f / 3.f : g == 3 ? 0.6f : 0.2f;
+                    const float s = wa * a.x + wb * b.x + wc * c.x, tt = wa * a.y + wb * b.y + wc * c.y;
+                    const float wr = (g == 0 ? -27.f / 48.f : 25.f / 48.f) * (oo + s * s + tt * tt);
+                    i0 += wr; is += wr * s; it += wr * tt;
+                }
+                m0 += (double)(at * i0); ms += (double)(at * is); mt += (double)(at * it);
+            }
+            const uint32_t ij = A.perm[__float_as_uint(reinterpret_cast<const float4*>(&A.faces[st + q])[1].w)];
+            const double wj = A.dtype == VT_F32 ? (double)((const float*)A.w)[ij] : ((const double*)A.w)[ij];
+            const double cf = (wk - wj) * (double)in1;
+            gx += cf * (m0 * o[0] + ms * u[0] + mt * w[0]);
+            gy += cf * (m0 * o[1] + ms * u[1] + mt * w[1]);
+            gz += cf * (m0 * o[2] + ms * u[2] + mt * w[2]);
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int s = CVT_LANES / 2; s; s >>= 1) {
+        gx += __shfl_xor_sync(0xffffffffu, gx, s);
+        gy += __shfl_xor_sync(0xffffffffu, gy, s);
+        gz += __shfl_xor_sync(0xffffffffu, gz, s);
+        fail = __shfl_xor_sync(0xffffffffu, (int)fail, s) || fail;
+    }
+    if (r != 0 || !in) return;
+    if (fail) {
+        const unsigned slot = atomicAdd(A.n_retry, 1u);
+        if (slot < A.retry_cap) A.retry[slot] = make_int4((int)k, 0, 0, 0);
+        else atomicAdd(A.n_fail, 1u);
+        return;
+    }
+    const CellOut co = A.cell[k];
+    const double s = -2.0 * wk * co.vol;
+    gx += s * co.zx; gy += s * co.zy; gz += s * co.zz;
+    if (A.dtype == VT_F32) {
+        float* out = (float*)A.out + 3 * (int64_t)ik;
+        out[0] = (float)gx; out[1] = (float)gy; out[2] = (float)gz;
+    } else {
+        double* out = (double*)A.out + 3 * (int64_t)ik;
+        out[0] = gx; out[1] = gy; out[2] = gz;
+    }
+}
+
+// A listed cell (a facet of more than PGON corners): one thread rebuilds it from its facet planes, its facets' vertices
+// ordered by angle in the facet plane and fanned.
+template <typename P, class CL>
 __global__ void __launch_bounds__(128) k_cvt_weighted(CvtArgs A) {
-    const int64_t n = RETRY ? (int64_t)min(*((volatile unsigned*)A.n_retry), A.retry_cap) : A.N;
+    const int64_t n = (int64_t)min(*((volatile unsigned*)A.n_retry), A.retry_cap);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = RETRY ? (int64_t)A.retry[e].x : e;
+        const int64_t k = (int64_t)A.retry[e].x;
         const P pi = ((const P*)A.spos)[k];
         GridArgs ga;
         ga.geo = A.geo; ga.faces = A.faces; ga.face_start = A.face_start; ga.face_count = A.face_count;
         CL C;
         const int f = grid_cell<P, CL>(C, ga, k, pi);
         if (f) {
-            if (!RETRY) {
-                const unsigned slot = atomicAdd(A.n_retry, 1u);
-                if (slot < A.retry_cap) A.retry[slot] = make_int4((int)k, 0, 0, 0);
-                else atomicAdd(A.n_fail, 1u);
-            } else {
-                atomicAdd(A.n_fail, 1u);
-            }
+            atomicAdd(A.n_fail, 1u);
             continue;
         }
         const uint32_t ik = A.perm[k];
@@ -1207,22 +1355,22 @@ int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g
 }
 
 int launch_cvt_weighted(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
-                        const uint32_t* face_start, const uint16_t* face_count, const CellOut* cell,
+                        const uint32_t* face_start, const uint16_t* face_count, const CellOut* cell, const float* rad,
                         const uint32_t* perm, const void* w, void* out, int4* retry, unsigned retry_cap,
                         unsigned* counters, int sm_count, cudaStream_t s) {
     CvtArgs a;
     a.spos = spos; a.N = N; a.geo = g; a.faces = faces; a.face_start = face_start; a.face_count = face_count;
-    a.cell = cell; a.perm = perm; a.w = w; a.dtype = dtype; a.out = out; a.retry = retry; a.retry_cap = retry_cap;
+    a.cell = cell; a.rad = rad; a.perm = perm; a.w = w; a.dtype = dtype; a.out = out; a.retry = retry; a.retry_cap = retry_cap;
     a.n_retry = counters; a.n_fail = counters + 1;
     cudaMemsetAsync(counters, 0, 16 * sizeof(unsigned), s);
-    const unsigned nb = (unsigned)((N + 127) / 128);
+    const unsigned nb = (unsigned)((N + 128 / CVT_LANES - 1) / (128 / CVT_LANES));
     const unsigned rb = (unsigned)(sm_count * 4);
     if (dtype == VT_F32) {
-        k_cvt_weighted<float4, TCell, false><<<nb, 128, 0, s>>>(a);
-        k_cvt_weighted<float4, TCellBig, true><<<rb, 128, 0, s>>>(a);
+        k_cvt_facets<float4><<<nb, 128, 0, s>>>(a);
+        k_cvt_weighted<float4, TCellBig><<<rb, 128, 0, s>>>(a);
     } else {
-        k_cvt_weighted<dpt4, TCell, false><<<nb, 128, 0, s>>>(a);
-        k_cvt_weighted<dpt4, TCellBig, true><<<rb, 128, 0, s>>>(a);
+        k_cvt_facets<dpt4><<<nb, 128, 0, s>>>(a);
+        k_cvt_weighted<dpt4, TCellBig><<<rb, 128, 0, s>>>(a);
     }
     return 2;
 }
