@@ -804,7 +804,7 @@ int vt_grid_density(vt_handle h, int G, int S, void* grid) {
     int rc = ensure_density(h);
     if (rc) return rc;
     h->n_launches += launch_grid(h->spos, h->dtype, h->N, h->geo, h->faces, h->face_start, h->face_count, h->keys,
-                                 h->dens_sorted, h->perm, G, S, grid, h->dstat, h->stream);
+                                 h->dens_sorted, h->perm, G, S, grid, h->stream);
     return cuda_rc(cudaGetLastError());
 }
 
