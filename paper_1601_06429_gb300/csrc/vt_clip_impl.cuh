@@ -51,7 +51,6 @@ struct Cap {
     static constexpr int CAND = 256;                      // candidates per radius pass
     static constexpr int STACK = TP <= 4 ? STACK_CAP : 4 * STACK_CAP;
 };
-constexpr int CHUNK = 4;
 // From this radius pass on (from the second one for listed cells) a search also tests nodes and points against the balls
 // of the cell's vertices: the cells that get there bound a void beside dense halos, and without it collect thousands of
 // halo points in passes of 256.
@@ -1645,15 +1644,16 @@ __global__ void __launch_bounds__(WPB * 32) k_clip(ClipArgs A) {
     for (;;) {
         uint32_t base = 0;
         const bool listed = !EXACT && A.warp_list != nullptr;
-        // (a list holds the cells other kernels gave up: the widest ones, one at a time)
-        const unsigned chunk = EXACT || listed ? 1u : (unsigned)CHUNK;
-        if (lane == 0) base = atomicAdd(EXACT ? &A.st->work_next_exact : &A.st->work_next, chunk);
+        // one cell at a time: a warp needs about 0.1 ms for it, so the counter is no burden, and with several in a row most
+        // warps go without work in a small set (four in a row: 1000 points 503 us, 280 one by one; 4096 FP64 points 1685
+        // and 726)
+        if (lane == 0) base = atomicAdd(EXACT ? &A.st->work_next_exact : &A.st->work_next, 1u);
         base = __shfl_sync(0xffffffffu, base, 0);
         uint32_t lim = EXACT ? *((volatile unsigned*)&A.st->n_exact_cells)
                              : listed ? *((volatile unsigned*)&A.st->n_warp_cells) : total;
         if (base >= lim) break;
-        for (uint32_t q = base; q < base + chunk && q < lim; q++) {
-            uint32_t self = EXACT ? A.exact_list[q] : listed ? A.warp_list[q] : q;
+        {
+            uint32_t self = EXACT ? A.exact_list[base] : listed ? A.warp_list[base] : base;
             VT_T0(tall);
             const unsigned f64_before = cc.n_fp64;
             // one call site (the cell routine is inlined once): the small start box first, then, if the cell
