@@ -337,9 +337,72 @@ size_t radix_tmp_bytes(int64_t N) {
     return 2 * h * sizeof(uint32_t) + scan_tmp_bytes((int64_t)h) + 256;
 }
 
-// sorts (key, val) by the low `bits` bits of key; the result ends in key/val
+// ---------------------------------------------------------------- sort of a small set
+// Six radix passes are eighteen dependent launches of a few blocks, 3 to 16 us each whatever the size.  A small set is
+// sorted in two: blocks sort runs of 1024 keys (bitonic, one key a thread; strides below a warp by shuffle), then every
+// key finds its place by binary searches in the other runs.  The key's index in the low 16 bits makes the order the
+// radix sort's (stable) one.  What bounds both is latency: 55 exchange stages, then 11 dependent cached loads a run.
+constexpr int SS_RUN = 1024;
+// the index has to fit into 16 bits; at 65536 points two thirds of the time is the search of the 63 other runs (70 us; radix
+// passes 168), at 1000 points 26 us instead of 112 (key, sort, gather and tree together)
+constexpr int64_t SS_MAX = 65536;
+
+__global__ void __launch_bounds__(SS_RUN) k_sort_runs(const uint64_t* __restrict__ key, int64_t N, uint64_t* __restrict__ out) {
+    __shared__ uint64_t buf[2][SS_RUN];
+    const int t = threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * SS_RUN + t;
+    uint64_t v = i < N ? (key[i] << 16) | (uint64_t)i : ~0ull;
+    int b = 0;
+#pragma unroll 1
+    for (int k = 2; k <= SS_RUN; k <<= 1) {
+        const bool up = (t & k) == 0;
+#pragma unroll 1
+        for (int j = k >> 1; j >= 32; j >>= 1) {
+            buf[b][t] = v;
+            __syncthreads();
+            const uint64_t o = buf[b][t ^ j];
+            b ^= 1;  // the next stage's writes go to the other buffer: one barrier a stage
+            v = (((t & j) == 0) == up) == (v < o) ? v : o;
+        }
+#pragma unroll 1
+        for (int j = min(k >> 1, 16); j > 0; j >>= 1) {
+            const uint64_t o = __shfl_xor_sync(0xffffffffu, v, j);
+            v = (((t & j) == 0) == up) == (v < o) ? v : o;
+        }
+    }
+    if (i < N) out[i] = v;
+}
+
+__global__ void __launch_bounds__(128) k_merge_runs(const uint64_t* __restrict__ runs, int64_t N, uint64_t* __restrict__ key,
+                                                    uint32_t* __restrict__ val) {
+    const int64_t t = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (t >= N) return;
+    const uint64_t v = runs[t];
+    const int own = (int)(t / SS_RUN), nr = (int)((N + SS_RUN - 1) / SS_RUN);
+    uint32_t rank = (uint32_t)(t - (int64_t)own * SS_RUN);
+#pragma unroll 4
+    for (int r = 0; r < nr; r++) {
+        const uint64_t* a = runs + (int64_t)r * SS_RUN;
+        const int len = (int)min((int64_t)SS_RUN, N - (int64_t)r * SS_RUN);
+        int p = 0;
+#pragma unroll
+        for (int h = SS_RUN; h > 0; h >>= 1)
+            if (p + h <= len && a[p + h - 1] < v) p += h;
+        if (r != own) rank += (uint32_t)p;
+    }
+    key[rank] = v >> 16;
+    val[rank] = (uint32_t)(v & 0xffffu);
+}
+
+// sorts (key, val) by the low `bits` bits of key, val[i] being i at the start; the result ends in key/val
 int radix_sort(uint64_t* key, uint32_t* val, uint64_t* key_alt, uint32_t* val_alt, int64_t N, int bits, void* tmp,
                cudaStream_t s) {
+    if (bits <= 48 && N <= SS_MAX) {
+        if (N == 0) return 0;
+        k_sort_runs<<<(unsigned)((N + SS_RUN - 1) / SS_RUN), SS_RUN, 0, s>>>(key, N, key_alt);
+        k_merge_runs<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(key_alt, N, key, val);
+        return 2;
+    }
     int nb = (int)((N + RS_TILE - 1) / RS_TILE);
     if (nb == 0) return 0;
     int launches = 0;
