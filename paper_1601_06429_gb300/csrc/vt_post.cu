@@ -152,8 +152,9 @@ int launch_nbr_emit(const Face* faces, const uint32_t* face_start, const uint16_
     return 1;
 }
 
-// A float as a double by integer arithmetic: the conversion instruction runs at the FP64 rate, 1/64 of the FP32 one.  Zeros
-// and denormals, which the shift would misplace, infinities and NaN take the conversion.
+// Facet records are FP32 and the sums over them FP64, which runs at 1/64 of the FP32 rate: what bounds the gradient
+// kernels is the count of FP64 instructions.  A float as a double by integer arithmetic (the conversion instruction runs
+// at the FP64 rate too); zeros and denormals, which the shift would misplace, and the rest take the same bits as a cast.
 __device__ __forceinline__ double f2d(float v) {
     const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
     if (m < 0x00800000u || m >= 0x7f800000u) return (double)v;
@@ -179,7 +180,7 @@ __global__ void k_gradient(const Face* __restrict__ faces, const uint32_t* __res
         double dr = dens[f.nbr] - ri;
         mxx = fmaf(f.dx, f.dx, mxx); mxy = fmaf(f.dx, f.dy, mxy); mxz = fmaf(f.dx, f.dz, mxz);
         myy = fmaf(f.dy, f.dy, myy); myz = fmaf(f.dy, f.dz, myz); mzz = fmaf(f.dz, f.dz, mzz);
-        bx = fma((double)f.dx, dr, bx); by = fma((double)f.dy, dr, by); bz = fma((double)f.dz, dr, bz);
+        bx = fma(f2d(f.dx), dr, bx); by = fma(f2d(f.dy), dr, by); bz = fma(f2d(f.dz), dr, bz);
     }
     double a = mxx, b = mxy, c = mxz, d = myy, e = myz, ff = mzz;
     double c00 = d * ff - e * e, c01 = c * e - b * ff, c02 = b * e - c * d;
@@ -210,12 +211,33 @@ int launch_gradient(const Face* faces, const uint32_t* face_start, const uint16_
     return 1;
 }
 
+// a / |(x, y, z)| to 1e-13 (results in FP32 only: they are the same ones), in FP32 but for the last sum: the FP32 reciprocal root s, the residual e = 1 - d^2 s^2 of it
+// with d^2 and s^2 as unevaluated sums of two floats, and 1/|d| = s (1 + e/2 + 3/8 e^2) to third order in e < 1e-6
+__device__ __forceinline__ double over_dist(float a, float x, float y, float z) {
+    const float xx = x * x, yy = y * y, zz = z * z;
+    const float s1 = __fadd_rn(xx, yy), b1 = __fsub_rn(s1, xx);
+    const float d2 = __fadd_rn(s1, zz), b2 = __fsub_rn(d2, s1);
+    if (!(d2 > 1e-26f && d2 < 1e26f)) {  // outside, the low parts would leave the range of a float
+        const double X = x, Y = y, Z = z;
+        return (double)a / sqrt(fma(Z, Z, fma(Y, Y, X * X)));
+    }
+    const float t1 = __fadd_rn(__fsub_rn(xx, __fsub_rn(s1, b1)), __fsub_rn(yy, b1));
+    const float t2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(d2, b2)), __fsub_rn(zz, b2));
+    const float lo = ((fmaf(x, x, -xx) + fmaf(y, y, -yy)) + fmaf(z, z, -zz)) + (t1 + t2);
+    const float s = rsqrtf(d2), ss = s * s, sl = fmaf(s, s, -ss);
+    const float e = fmaf(-lo, ss, fmaf(-d2, sl, fmaf(-d2, ss, 1.f)));
+    const float p = a * s;
+    return f2d(p) + f2d(fmaf(p, e * fmaf(0.375f, e, 0.5f), fmaf(a, s, -p)));
+}
+
 // ------------------------------------------------------------------ Green-Gauss gradient
 // grad rho_i = (1/V_i) sum_f A_f (rho_j - rho_i) c_f / |d_f| over the facets between particles, c_f the facet
 // centroid relative to x_i and d_f the neighbour image's displacement: the surface integral of rho n over the
 // cell with rho at a facet centroid interpolated linearly between the two sites, exact for a linear field
 // (the tangential parts cancel on a closed Voronoi cell); on a box wall rho is taken as rho_i.  One thread per
-// cell, FP64 sums over FP32 facet records.
+// cell, FP64 sums over FP32 facet records: six FP64 instructions a facet (FP32 results), and the gathers of records and
+// densities, bound it (one million clustered cells: 522 us; 1465 us with an FP64 root and quotient a facet).  FP64 results
+// keep the FP64 root and quotient.
 template <typename T>
 __global__ void k_gradient_gg(const Face* __restrict__ faces, const uint32_t* __restrict__ face_start,
                               const uint16_t* __restrict__ face_count, const CellOut* __restrict__ cell,
@@ -229,11 +251,16 @@ __global__ void k_gradient_gg(const Face* __restrict__ faces, const uint32_t* __
     double gx = 0.0, gy = 0.0, gz = 0.0;
     for (int q = 0; q < cnt; q++) {
         const Face f = faces[st + q];
-        const double r = sqrt(fma((double)f.dz, (double)f.dz, fma((double)f.dy, (double)f.dy, (double)f.dx * f.dx)));
-        const double w = (double)f.area * (dens[f.nbr] - ri) / r;
-        gx = fma(w, (double)f.cx, gx);
-        gy = fma(w, (double)f.cy, gy);
-        gz = fma(w, (double)f.cz, gz);
+        const double dr = dens[f.nbr] - ri;
+        double w;
+        if (sizeof(T) == 4) w = over_dist(f.area, f.dx, f.dy, f.dz) * dr;
+        else {
+            const double x = f.dx, y = f.dy, z = f.dz;
+            w = (double)f.area * dr / sqrt(fma(z, z, fma(y, y, x * x)));
+        }
+        gx = fma(w, f2d(f.cx), gx);
+        gy = fma(w, f2d(f.cy), gy);
+        gz = fma(w, f2d(f.cz), gz);
     }
     const double iv = 1.0 / cell[k].vol;
     const uint32_t i = perm[k];
