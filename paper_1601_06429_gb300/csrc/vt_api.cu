@@ -321,10 +321,10 @@ int vt_default_params(vt_params* p) {
 namespace {
 
 // Threads per cell where the caller leaves the choice to the library (0).  FP32 filter: 4 lanes a cell from 65,536
-// particles on, where the chip has enough cells for 8 of them to share a warp; clipping at 32,768 / 65,536 / 2,097,152
-// uniform points takes 1.94 / 3.48 / 114.5 ms by a warp a cell and 1.65 / 2.47 / 40.2 ms by 4 lanes, at 32,768 /
-// 65,536 / 150,000 / 2,097,152 clustered points 3.21 / 6.17 / 12.4 / 128 ms and 4.84 / 6.76 / 8.8 / 61.4 ms (8 lanes
-// are slower than 4 at every size).
+// particles on, where the chip has enough cells for 8 of them to share a warp; clipping 40,000 / 65,536 / 100,000 /
+// 2,097,152 uniform points takes 1.98 / 3.18 / 4.95 / 114.5 ms by a warp a cell and 1.69 / 2.30 / 2.88 / 40.2 ms by 4
+// lanes, 65,537 / 100,000 / 200,000 / 2,097,152 clustered points 4.72 / 6.76 / 13.1 / 128 ms and 5.27 / 5.99 / 9.08 /
+// 61 ms (8 lanes are slower than 4 at every size).
 constexpr int64_t GROUP_MIN_N = 65536;
 int default_tpc(int precision, int64_t N) { return precision == VT_FILTER32 && N >= GROUP_MIN_N ? 4 : 32; }
 

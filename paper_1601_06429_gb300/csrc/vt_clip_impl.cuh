@@ -1745,7 +1745,7 @@ static void launch_one_t(const ClipArgs& a, int sm_count, cudaStream_t s) {
 template <typename P, typename CT, bool EXACT>
 static void launch_one(const ClipArgs& a, int sm_count, cudaStream_t s) {
     // searches against the vertices' balls: for listed cells and larger sets.  Below 8192 particles no halo holds enough
-    // points to make a cell's search long, and the extra code costs 3 % (505 -> 521 us at 1000 uniform points)
+    // points to make a cell's search long, and the extra code costs 3 % of a call with 1000 uniform points
     if (EXACT || (!a.warp_list && a.N <= 8192)) {
         if (a.sset) launch_one_t<P, CT, EXACT, true, false>(a, sm_count, s);
         else launch_one_t<P, CT, EXACT, false, false>(a, sm_count, s);

@@ -166,7 +166,7 @@ extern "C" int vt_volumes_noalloc(const void* pos, int dtype, int64_t N, const d
     a.st = dstat;
     a.xws = xws;
     a.xws_warps = kExactWarps;
-    a.warp_list = nullptr;  // the warp-per-cell kernel on every cell, as vt_build's default
+    a.warp_list = nullptr;  // the warp-per-cell kernel on every cell, as vt_build's default at these sizes
     launch_clip(a, nullptr, dtype, VT_FILTER32, sms, s);
     launch_clip_exact(a, dtype, sms, s);
     rc = rc_of(cudaGetLastError());
