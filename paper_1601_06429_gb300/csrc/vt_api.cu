@@ -844,7 +844,7 @@ int vt_grid_density_volume(vt_handle h, int G, void* grid) {
     rc = ensure_retry(h);
     if (rc) return rc;
     h->n_launches += launch_grid_volume(h->spos, h->dtype, h->N, h->geo, h->faces, h->face_start, h->face_count,
-                                        h->dens_sorted, h->rad, h->cell, h->exact_list, G, h->gacc, h->gretry, GRID_RETRY_CAP, h->gcnt, grid,
+                                        h->dens_sorted, h->rad, h->cell, h->exact_list, h->keys_alt, G, h->gacc, h->gretry, GRID_RETRY_CAP, h->gcnt, grid,
                                         h->sm_count, h->stream);
     return cuda_rc(cudaGetLastError());
 }

@@ -1576,12 +1576,15 @@ int launch_group(const ClipArgs& a, const GroupBuf& b, int sm_count, cudaStream_
 // meet.  The pairs that some plane crosses wait in queues (of about the same number of crossing planes) until there are
 // enough, and are cut by the crossing planes alone, G lanes a pair as in k_group_clip, starting from the voxel's box (cut
 // down to the ball's).  Sides are plain FP32 signs: a wrong sign within rounding of a plane moves a rounding-sized sliver.
-// Cells whose balls meet more than GV_BIG voxels are listed and a second launch spreads each over all warps.
+// Cells whose balls meet more than GV_BIG voxels are listed, with the running count of their units of GV_BIG pairs, and
+// the warps of a second launch take those units from a counter (2,097,152 clustered particles on 256^3 voxels: 166 ms;
+// 8.1 s when every warp went through all listed cells, 6.9 s with one thread a cell).
 // Bound by instruction issue, as k_group_clip.  131,072 clustered particles on 32^3 voxels: 4.7 ms; 297 ms with one thread
 // walking all voxels of a cell and clipping a copy of it by each voxel's walls; 13 ms with one thread a pair (5 of 32 lanes
 // active, and the lanes' polytopes in local memory).
 constexpr int GV_BIG = 512;
 constexpr int GV_CLASSES = 4;
+constexpr int BIG_BITS = 36;
 
 struct GridWarp {
     int pref[33];
@@ -1601,7 +1604,8 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
     GCell& C = cells[gsh / G];
     const P* const spos = (const P*)A.spos;
     const double vox = A.h[0] * A.h[1] * A.h[2];
-    const unsigned n_big = BIG ? *((volatile unsigned*)A.n_big) : 0u;
+    const unsigned long long listed = BIG ? *((volatile unsigned long long*)A.n_big) : 0ull;
+    const unsigned long long n_units = listed & ((1ull << BIG_BITS) - 1ull);
     auto gballot = [&](bool p) -> unsigned { return (__ballot_sync(FULL, p) >> gsh) & GM; };
     auto gsum = [&](float v) -> float {
 #pragma unroll
@@ -1612,7 +1616,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
 #pragma unroll
     for (int c = 0; c < GV_CLASSES; c++) nq[c] = 0;
 
-    unsigned e = 0, b = 0;
+    unsigned b = 0;
     int64_t total = 0, t1 = 0;
     bool more = true;
     for (;;) {
@@ -1620,9 +1624,18 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
         if (t1 >= total && more) {
             total = 0;
             if (BIG) {
-                // one listed cell over all warps
-                if (e >= n_big) more = false;
+                // one unit of a listed cell: the last cell whose first unit is not beyond it
+                unsigned long long u = 0;
+                if (lane == 0) u = atomicAdd(A.big_queue, 1ull);
+                u = __shfl_sync(FULL, u, 0);
+                if (u >= n_units) more = false;
                 else {
+                    uint32_t e = 0, e1 = (uint32_t)(listed >> BIG_BITS);
+                    while (e1 - e > 1) {
+                        const uint32_t mid = (e + e1) >> 1;
+                        if (A.big_unit[mid] <= u) e = mid;
+                        else e1 = mid;
+                    }
                     const uint32_t k = A.big[e];
                     const P pi = spos[k];
                     const double xi[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
@@ -1633,8 +1646,8 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                         S.n[lane][0] = lane == 0 ? n[0] : lane == 1 ? n[1] : n[2];
                     }
                     b = k;
-                    e++;
-                    t1 = (int64_t)blockIdx.x * 32;
+                    t1 = (int64_t)(u - A.big_unit[e]) * GV_BIG;
+                    total = min(total, t1 + GV_BIG);
                 }
             } else {
                 if (lane == 0) b = atomicAdd(A.queue, 32u);
@@ -1656,7 +1669,10 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                             }
                             atomicAdd(&A.acc[(v[2] * A.G + v[1]) * A.G + v[0]], A.dens[k] * A.cell[k].vol);
                         } else if (mm > GV_BIG) {
-                            A.big[atomicAdd(A.n_big, 1u)] = (uint32_t)k;
+                            const unsigned long long o =
+                                atomicAdd(A.n_big, (1ull << BIG_BITS) + (unsigned long long)((mm + GV_BIG - 1) / GV_BIG));
+                            A.big[o >> BIG_BITS] = (uint32_t)k;
+                            A.big_unit[o >> BIG_BITS] = o & ((1ull << BIG_BITS) - 1ull);
                         } else {
                             m = (int)mm;
                             for (int c = 0; c < 3; c++) { S.a0[c][lane] = a0[c]; S.n[c][lane] = n[c]; }
@@ -1707,7 +1723,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                 if (cls == c) S.q[c][nq[c] + __popc(cm & lt)] = ent;
                 nq[c] += __popc(cm);
             }
-            t1 += BIG ? (int64_t)gridDim.x * 32 : 32;
+            t1 += 32;
             __syncwarp();
         }
         // ---------------------------------------------------------------- eight pairs of a class, while one is full

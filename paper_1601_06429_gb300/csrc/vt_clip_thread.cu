@@ -1328,7 +1328,7 @@ __global__ void k_grid_finish(const double* __restrict__ acc, int64_t n, double 
 
 int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
                        const uint32_t* face_start, const uint16_t* face_count, const double* dens_sorted, const float* rad,
-                       const CellOut* cell, uint32_t* big, int G, double* acc, int4* retry, unsigned retry_cap, unsigned* counters, void* out, int sm_count,
+                       const CellOut* cell, uint32_t* big, uint64_t* big_unit, int G, double* acc, int4* retry, unsigned retry_cap, unsigned* counters, void* out, int sm_count,
                        cudaStream_t s) {
     GridArgs a;
     a.spos = spos; a.N = N; a.geo = g; a.faces = faces; a.face_start = face_start; a.face_count = face_count;
@@ -1338,8 +1338,10 @@ int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g
     const int64_t n = (int64_t)G * G * G;
     cudaMemsetAsync(acc, 0, n * sizeof(double), s);
     cudaMemsetAsync(counters, 0, 16 * sizeof(unsigned), s);
-    a.rad = rad; a.cell = cell; a.big = big;
-    a.n_big = counters + 2; a.queue = counters + 3;
+    a.rad = rad; a.cell = cell; a.big = big; a.big_unit = big_unit;
+    a.queue = counters + 2;
+    a.n_big = reinterpret_cast<unsigned long long*>(counters + 4);
+    a.big_queue = reinterpret_cast<unsigned long long*>(counters + 6);
     launch_grid_pairs(a, dtype, sm_count, s);
     const unsigned rb = (unsigned)(sm_count * 4);
     if (dtype == VT_F32) {

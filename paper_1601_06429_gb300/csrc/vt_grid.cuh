@@ -14,8 +14,10 @@ struct GridArgs {
     const double* dens;  // sorted order
     const float* rad;    // bound of each cell's radius
     const CellOut* cell;
-    uint32_t* big;       // cells whose ball meets more than GV_BIG voxels
-    unsigned* n_big;
+    uint32_t* big;       // cells whose ball meets more than GV_BIG voxels, and the first unit of work of each
+    uint64_t* big_unit;
+    unsigned long long* n_big;  // listed cells above bit BIG_BITS, their units of GV_BIG pairs below
+    unsigned long long* big_queue;
     unsigned* queue;
     int G;
     double h[3];         // voxel side L / G

@@ -117,7 +117,8 @@ int launch_cvt_weighted(const void* spos, int dtype, int64_t N, const Geometry& 
                         unsigned* counters, int sm_count, cudaStream_t s);
 int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
                        const uint32_t* face_start, const uint16_t* face_count, const double* dens_sorted, const float* rad,
-                       const CellOut* cell, uint32_t* big, int G, double* acc, int4* retry, unsigned retry_cap, unsigned* counters, void* out, int sm_count,
+                       const CellOut* cell, uint32_t* big, uint64_t* big_unit, int G, double* acc, int4* retry, unsigned retry_cap,
+                       unsigned* counters, void* out, int sm_count,
                        cudaStream_t s);
 int launch_gradient_gg(const Face* faces, const uint32_t* face_start, const uint16_t* face_count, const CellOut* cell,
                        const double* dens_sorted, const uint32_t* perm, int64_t N, void* grad, int dtype,

@@ -29,6 +29,7 @@ def _lib():
     (12, 40, False, np.float64),      # a cell covers thousands of voxels
     (300, 13, True, np.float32), (300, 1, True, np.float32),
     (2500, 37, False, np.float32), (2500, 2, True, np.float64),
+    (300, 64, True, np.float32),      # every cell over more voxels than one unit of work, the units not full
     (9000, 5, True, np.float32)])
 def test_voxel_averages(n, G, periodic, dtype, oracle_mod):
     x = inputs.uniform(n, seed=n + G, dtype=np.float32).astype(dtype)
