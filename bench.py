@@ -51,10 +51,10 @@ WORK = {
     "clustered16M": {"n_cert": 163.17, "verts": 26.74, "faces": 15.37},
     "halosets4096": {"n_cert": 147.19, "verts": 26.55, "faces": 15.27},
 }
-# DRAM bytes (read + write) of one launch of the clipping kernel: dram__bytes_read.sum + dram__bytes_write.sum of
-# one launch on the 2,097,152-point clustered set (543 B per cell, profiles/k_clip_clustered2M_dram.md) times the
-# cells of the launch (the facet records that dominate it grow with the cells)
-CLIP_TRAFFIC_PER_CELL = {"filter32": 543.3}
+# DRAM bytes (read + write) of one step's clipping kernels (the lane groups' passes and the warp kernel's list):
+# dram__bytes_read.sum + dram__bytes_write.sum over their launches on the 2,097,152-point clustered set (4473 B per cell,
+# profiles/k_group_clustered2M_dram.md) times the cells of the step (a larger set runs as chunks of that size)
+CLIP_TRAFFIC_PER_CELL = {"filter32": 4472.6}
 CLIP_TRAFFIC = {("clustered16M", "filter32"): CLIP_TRAFFIC_PER_CELL["filter32"] * 16777216,
                 ("clustered2M", "filter32"): CLIP_TRAFFIC_PER_CELL["filter32"] * 2097152}
 # FMA lanes per SM of the GB300 (sm_103): 128 FP32; the FP64 rate is 1/64 of it (2 FP64 FMA per clock per SM)
@@ -610,7 +610,8 @@ def run_ours(args):
             "gpu_launches": launches,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": CLIP_TRAFFIC.get((args.workload, args.precision)),
-                         "kernel": "k_clip (clipping, security test, facet emission)",
+                         "kernel": ("k_group_search, k_group_clip, k_clip" if args.precision == "filter32" else "k_clip")
+                                   + " (clipping, security test, facet emission)",
                          "work": "%.0f algorithmic flops/cell x %d cells per launch" % (fpc, N),
                          "peak_note": "%s FMA issue: %d SMs x %d lanes x 2 flop x %.0f MHz (derived)"
                                       % ("FP32" if args.precision == "filter32" else "FP64", sm_count,
