@@ -591,6 +591,8 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
                             int nc = __shfl_sync(FULL, n, c);
 #pragma unroll 1
                             for (int tries = 0; nc + __popc(hm) > GNC; tries++) {
+                                // other lanes' entries of the leaves since the last barrier (a vote does not order them)
+                                __syncwarp();
                                 // a full list: the part nearer than the mean of it stays, and the pass ends there
                                 int sum = 0;
                                 for (int i = (int)lane; i < nc; i += 32) sum += S.ck[c][i];
