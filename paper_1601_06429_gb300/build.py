@@ -17,7 +17,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libvt_gb300.so")
 SOURCES = ["vt_api.cu", "vt_sort.cu", "vt_post.cu", "vt_clip_f32.cu", "vt_clip_f64.cu", "vt_clip_exact.cu",
            "vt_clip_thread.cu", "vt_clip_group.cu", "vt_noalloc.cu"]
-HEADERS = ["vt_internal.cuh", "vt_kernels.cuh", "vt_clip_impl.cuh", "vt_grid.cuh"]
+HEADERS = ["vt_internal.cuh", "vt_kernels.cuh", "vt_clip_impl.cuh", "vt_grid.cuh", "vt_polytope.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

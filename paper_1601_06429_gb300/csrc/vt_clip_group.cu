@@ -27,6 +27,7 @@
 
 #include "vt_clip_impl.cuh"
 #include "vt_grid.cuh"
+#include "vt_polytope.cuh"
 
 namespace vt {
 namespace {
@@ -64,10 +65,11 @@ struct __align__(16) GCell {
         struct {
             uint32_t bnd[GBND];              // boundary edges of a cut (x, y, kept slot, its edge, new slot)
             uint8_t lnk_s[GNP], lnk_e[GNP];  // new vertex whose boundary edge starts / ends at a plane
+            uint8_t lnk_n[GNP];              // the plane at which the boundary edge that starts at a plane ends
         };
         uint32_t first[GNP];                 // emission: a plane's first slot
     };
-    uint32_t pad[6];
+    uint32_t pad[4];
 };
 static_assert(sizeof(GCell) % 32 == 16, "an odd number of 16-byte units: reads of one slot of every cell do not conflict");
 static_assert(offsetof(GCell, bnd) <= GROUP_STATE && GROUP_STATE % 16 == 0, "the state kept between passes: V, Pl, Ad, Ps, Sq");
@@ -739,12 +741,55 @@ __global__ void __launch_bounds__(SWARPS * 32, 8) k_group_search(const __grid_co
     }
 }
 
+// The vertices of `in` reached from `seed` over edges within it, and the removed side of a cut by pl made whole, with the
+// kept side (vt_polytope.cuh): what is apart from the vertex farthest out is kept, what is then apart from the vertex farthest in
+// is removed.  One lane's work, for the few cuts whose signs contradict each other.
+__device__ unsigned long long reach_of_slots(const GCell& C, int seed, unsigned long long in) {
+    unsigned long long got = 1ull << seed, front = got;
+    while (front) {
+        unsigned long long to = 0ull;
+        for (; front; front &= front - 1ull) {
+            const uint32_t ad = C.Ad[__ffsll((long long)front) - 1];
+            to |= (1ull << (ad & 63u)) | (1ull << ((ad >> 8) & 63u)) | (1ull << ((ad >> 16) & 63u));
+        }
+        front = to & in & ~got;
+        got |= front;
+    }
+    return got;
+}
+__device__ __noinline__ unsigned long long whole_sides(const GCell& C, float4 pl, unsigned long long all, unsigned long long rem) {
+    float so = -INFINITY, si = INFINITY;
+    int far_out = 0, far_in = 0;
+    for (unsigned long long m = all; m; m &= m - 1ull) {
+        const int s = __ffsll((long long)m) - 1;
+        const float4 v = C.V[s];
+        const float d = beyond(pl, v.x, v.y, v.z);
+        if ((rem >> s) & 1ull) {
+            if (d > so) { so = d; far_out = s; }
+        } else if (d < si) {
+            si = d;
+            far_in = s;
+        }
+    }
+    rem = reach_of_slots(C, far_out, rem);
+    return all & ~reach_of_slots(C, far_in, all & ~rem);
+}
+
 // Cut the cells of the groups with `cut` set by the plane that lane `src` of the group holds (pl, from its lane's particle
 // `from`), which removes exactly the vertex slots rem: the plane gets an id, every edge between a removed and a kept vertex
 // becomes a new vertex (w: the new slots).  fail is set where the cell outgrows its capacity or a vertex is
-// ill-conditioned.  The whole warp calls.
-template <int G>
-__device__ __forceinline__ void group_cut(GCell& C, bool& cut, int src, unsigned rem0, unsigned rem1, float4 pl, uint32_t from,
+// ill-conditioned.  SIGNS: rem comes from plain signs, which may contradict each other; where the boundary is not one loop
+// that meets a plane once, both sides are made whole first and rem returns what was removed; and new vertices are taken on
+// their edges.  The whole warp calls.
+constexpr int EARLY = 3;  // new vertices a lane holds before it writes them (SIGNS)
+__device__ __forceinline__ float4 on_edge(const GCell& C, float4 pl, uint32_t p, uint32_t rec) {
+    const float4 a = C.V[rec >> 26], b = C.V[(rec >> 12) & 63u];
+    const float e = edge_part(beyond(pl, a.x, a.y, a.z), beyond(pl, b.x, b.y, b.z));
+    return make_float4(fmaf(e, b.x - a.x, a.x), fmaf(e, b.y - a.y, a.y), fmaf(e, b.z - a.z, a.z),
+                       pack_w(0.f, pack_ids(rec & 63u, (rec >> 6) & 63u, p)));
+}
+template <int G, bool SIGNS>
+__device__ __forceinline__ void group_cut(GCell& C, bool& cut, int src, unsigned& rem0, unsigned& rem1, float4 pl, uint32_t from,
                                           unsigned& vlo, unsigned& vhi, int& np, int& nseq, int& fail, unsigned& w0,
                                           unsigned& w1) {
     const unsigned lane = lane_id();
@@ -799,91 +844,141 @@ __device__ __forceinline__ void group_cut(GCell& C, bool& cut, int src, unsigned
         np++;
         nseq++;
     }
-    // boundary edges: edge k of a removed vertex whose neighbour across it is kept; numbered by chunk of
-    // 32 slots, edge, slot
     int nB = 0;
 #pragma unroll 1
-    for (int e = 0; e < 2; e++) {
-        const unsigned re = cut ? (e ? rem1 : rem0) : 0u;
-        if (!__any_sync(FULL, re != 0u)) continue;
-        unsigned first = re;
+    for (int tries = 0;; tries++) {
+        // boundary edges: edge k of a removed vertex whose neighbour across it is kept; numbered by chunk of
+        // 32 slots, edge, slot
+        nB = 0;
+#pragma unroll 1
+        for (int e = 0; e < 2; e++) {
+            const unsigned re = cut ? (e ? rem1 : rem0) : 0u;
+            if (!__any_sync(FULL, re != 0u)) continue;
+            unsigned first = re;
+#pragma unroll
+            for (int q = 0; q < G - 1; q++)
+                if (q < r) first &= first - 1u;
+            unsigned b0 = 0u, b1 = 0u, b2 = 0u;
+            unsigned mm = first;
+#pragma unroll 1
+            while (__any_sync(FULL, mm != 0u)) {
+                if (mm) {
+                    const unsigned bit = mm & (0u - mm);
+                    const uint32_t ad = C.Ad[e * 32 + __ffs(mm) - 1];
+                    if (!in_set(rem0, rem1, ad & 255u)) b0 |= bit;
+                    if (!in_set(rem0, rem1, (ad >> 8) & 255u)) b1 |= bit;
+                    if (!in_set(rem0, rem1, (ad >> 16) & 255u)) b2 |= bit;
+                }
+#pragma unroll
+                for (int q = 0; q < G; q++) mm &= mm - 1u;
+            }
+            b0 = gor<G>(b0); b1 = gor<G>(b1); b2 = gor<G>(b2);
+            const int n0 = __popc(b0), n1 = __popc(b1), n2 = __popc(b2);
+            mm = first;
+#pragma unroll 1
+            while (__any_sync(FULL, mm != 0u)) {
+                if (mm) {
+                    const unsigned bit = mm & (0u - mm);
+                    const uint32_t t = (uint32_t)(e * 32 + __ffs(mm) - 1);
+                    const uint32_t ad = C.Ad[t], tr = __float_as_uint(C.V[t].w);
+#pragma unroll
+                    for (int q = 0; q < 3; q++) {
+                        const unsigned bq = q == 0 ? b0 : q == 1 ? b1 : b2;
+                        if (!(bq & bit)) continue;
+                        const int o = nB + (q > 0 ? n0 : 0) + (q > 1 ? n1 : 0) + __popc(bq & (bit - 1u));
+                        const uint32_t nb = (ad >> (8 * q)) & 63u;
+                        const uint32_t na = C.Ad[nb];
+                        const uint32_t kn = (na & 255u) == t ? 0u : ((na >> 8) & 255u) == t ? 1u : 2u;
+                        const uint32_t x = (tr >> (IDB5 * q)) & IDM5, y = (tr >> (q == 2 ? 0 : IDB5 * (q + 1))) & IDM5;
+                        if (o < GBND) C.bnd[o] = x | (y << 6) | (nb << 12) | (kn << 18) | (SIGNS ? t << 26 : 0u);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < G; q++) mm &= mm - 1u;
+            }
+            nB += n0 + n1 + n2;
+        }
+        unsigned long long fr = ~((((unsigned long long)vhi << 32) | vlo) & ~(((unsigned long long)rem1 << 32) | rem0)) &
+                                (GNT == 64 ? ~0ull : (1ull << (GNT & 63)) - 1ull);
+        if (SIGNS && nB > EARLY * G) fr &= ~(((unsigned long long)rem1 << 32) | rem0);
+        const bool over = cut && (nB > min(GBND, __popcll(fr)) || nB < 3);
+        if (over && (!SIGNS || tries)) { fail = GF_CAP; cut = false; }
+        if (!cut) nB = 0;
+        __syncwarp();
+        // the i-th boundary edge takes the i-th lowest free slot
+        w0 = w1 = 0u;
 #pragma unroll
         for (int q = 0; q < G - 1; q++)
-            if (q < r) first &= first - 1u;
-        unsigned b0 = 0u, b1 = 0u, b2 = 0u;
-        unsigned mm = first;
+            if (q < r) fr &= fr - 1ull;
+        const int nl = over ? 0 : nB, nlmax = __reduce_max_sync(FULL, nl);
 #pragma unroll 1
-        while (__any_sync(FULL, mm != 0u)) {
-            if (mm) {
-                const unsigned bit = mm & (0u - mm);
-                const uint32_t ad = C.Ad[e * 32 + __ffs(mm) - 1];
-                if (!in_set(rem0, rem1, ad & 255u)) b0 |= bit;
-                if (!in_set(rem0, rem1, (ad >> 8) & 255u)) b1 |= bit;
-                if (!in_set(rem0, rem1, (ad >> 16) & 255u)) b2 |= bit;
+        for (int i = r; i < nlmax; i += G) {
+            if (i < nl) {
+                const uint32_t t = (uint32_t)__ffsll((long long)fr) - 1u;
+                const uint32_t rec = C.bnd[i];
+                C.lnk_s[rec & 63u] = (uint8_t)t;
+                C.lnk_e[(rec >> 6) & 63u] = (uint8_t)t;
+                if (SIGNS) C.lnk_n[rec & 63u] = (uint8_t)((rec >> 6) & 63u);
+                C.bnd[i] = rec | (t << 20);
+                if (t < 32) w0 |= 1u << t; else w1 |= 1u << (t - 32);
             }
 #pragma unroll
-            for (int q = 0; q < G; q++) mm &= mm - 1u;
+            for (int q = 0; q < G; q++) fr &= fr - 1ull;
         }
-        b0 = gor<G>(b0); b1 = gor<G>(b1); b2 = gor<G>(b2);
-        const int n0 = __popc(b0), n1 = __popc(b1), n2 = __popc(b2);
-        mm = first;
-#pragma unroll 1
-        while (__any_sync(FULL, mm != 0u)) {
-            if (mm) {
-                const unsigned bit = mm & (0u - mm);
-                const uint32_t t = (uint32_t)(e * 32 + __ffs(mm) - 1);
-                const uint32_t ad = C.Ad[t], tr = __float_as_uint(C.V[t].w);
-#pragma unroll
-                for (int q = 0; q < 3; q++) {
-                    const unsigned bq = q == 0 ? b0 : q == 1 ? b1 : b2;
-                    if (!(bq & bit)) continue;
-                    const int o = nB + (q > 0 ? n0 : 0) + (q > 1 ? n1 : 0) + __popc(bq & (bit - 1u));
-                    const uint32_t nb = (ad >> (8 * q)) & 63u;
-                    const uint32_t na = C.Ad[nb];
-                    const uint32_t kn = (na & 255u) == t ? 0u : ((na >> 8) & 255u) == t ? 1u : 2u;
-                    const uint32_t x = (tr >> (IDB5 * q)) & IDM5, y = (tr >> (q == 2 ? 0 : IDB5 * (q + 1))) & IDM5;
-                    if (o < GBND) C.bnd[o] = x | (y << 6) | (nb << 12) | (kn << 18);
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < G; q++) mm &= mm - 1u;
+        if (!SIGNS) break;
+        __syncwarp();
+        // one loop: from the first edge's plane on, back at it after nB steps and not before (an entry may be an older
+        // cut's, or never written: the steps are bounded)
+        bool bad = over;
+        if (nl > 0) {
+            const uint32_t x0 = C.bnd[0] & 63u;
+            uint32_t x = x0;
+            int k = 0;
+            do {
+                x = C.lnk_n[x];
+                k++;
+            } while (x != x0 && x < (uint32_t)GNP && k < nl);
+            bad = x != x0 || k != nl;
         }
-        nB += n0 + n1 + n2;
+        if (!__any_sync(FULL, bad)) break;
+        if (tries) {  // (both sides whole: not reached)
+            if (bad) { fail = GF_CAP; cut = false; nB = 0; }
+            break;
+        }
+        unsigned long long rem = ((unsigned long long)rem1 << 32) | rem0;
+        const float4 f = C.Pl[cut ? p : 0];
+        if (bad && r == 0) rem = whole_sides(C, f, ((unsigned long long)vhi << 32) | vlo, rem);
+        rem0 = __shfl_sync(FULL, (unsigned)rem, gsh);
+        rem1 = __shfl_sync(FULL, (unsigned)(rem >> 32), gsh);
+        __syncwarp();
     }
-    unsigned long long fr = ~((((unsigned long long)vhi << 32) | vlo) & ~(((unsigned long long)rem1 << 32) | rem0)) &
-                            (GNT == 64 ? ~0ull : (1ull << (GNT & 63)) - 1ull);
-    if (cut && (nB > min(GBND, __popcll(fr)) || nB < 3)) { fail = GF_CAP; cut = false; }
-    if (!cut) nB = 0;
-    __syncwarp();
-    // the i-th boundary edge takes the i-th lowest free slot
-    w0 = w1 = 0u;
-#pragma unroll
-    for (int q = 0; q < G - 1; q++)
-        if (q < r) fr &= fr - 1ull;
     const int nBmax = __reduce_max_sync(FULL, nB);
-#pragma unroll 1
-    for (int i = r; i < nBmax; i += G) {
-        if (i < nB) {
-            const uint32_t t = (uint32_t)__ffsll((long long)fr) - 1u;
-            const uint32_t rec = C.bnd[i];
-            C.lnk_s[rec & 63u] = (uint8_t)t;
-            C.lnk_e[(rec >> 6) & 63u] = (uint8_t)t;
-            C.bnd[i] = rec | (t << 20);
-            if (t < 32) w0 |= 1u << t; else w1 |= 1u << (t - 32);
-        }
-#pragma unroll
-        for (int q = 0; q < G; q++) fr &= fr - 1ull;
-    }
     __syncwarp();
+    if (SIGNS) {
+        // a new vertex may take the slot of a removed one that another lane reads: the first ones are read by all lanes before
+        // any is written, and a longer boundary keeps off the removed slots
+        float4 v[EARLY];
+#pragma unroll
+        for (int q = 0; q < EARLY; q++)
+            if (r + q * G < nB) v[q] = on_edge(C, C.Pl[p], (uint32_t)p, C.bnd[r + q * G]);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < EARLY; q++)
+            if (r + q * G < nB) C.V[(C.bnd[r + q * G] >> 20) & 63u] = v[q];
+    }
     bool ill = false;
 #pragma unroll 1
     for (int i = r; i < nBmax; i += G) {
         if (i < nB) {
             const uint32_t rec = C.bnd[i];
             const uint32_t x = rec & 63u, y = (rec >> 6) & 63u, nb = (rec >> 12) & 63u, kn = (rec >> 18) & 3u,
-                           t = rec >> 20;
+                           t = SIGNS ? (rec >> 20) & 63u : rec >> 20;
             C.Ad[t] = nb | ((uint32_t)C.lnk_s[y] << 8) | ((uint32_t)C.lnk_e[x] << 16);
             reinterpret_cast<uint8_t*>(&C.Ad[nb])[kn] = (uint8_t)t;
+            if (SIGNS) {
+                if (i >= EARLY * G) C.V[t] = on_edge(C, C.Pl[p], (uint32_t)p, rec);
+                continue;
+            }
             float rr;
             const float4 v = vertex_at(C, x, y, (uint32_t)p, rr);
             C.V[t] = make_float4(v.x, v.y, v.z, pack_w(v.w, pack_ids(x, y, (uint32_t)p)));
@@ -1127,11 +1222,11 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
                 bool cut = open && !fail && cm != 0u;
                 if (!__any_sync(FULL, cut)) break;
                 const int src = gsh + (cut ? __ffs(cm) - 1 : 0);
-                const unsigned rem0 = __shfl_sync(FULL, olo, src), rem1 = __shfl_sync(FULL, ohi, src);
+                unsigned rem0 = __shfl_sync(FULL, olo, src), rem1 = __shfl_sync(FULL, ohi, src);
                 unsigned w0, w1;
                 c_cut += cut && r == 0;
                 dirty += cut;
-                group_cut<G>(C, cut, src, rem0, rem1, make_float4(cdx, cdy, cdz, chh), cjj, vlo, vhi, np, nseq, fail, w0, w1);
+                group_cut<G, false>(C, cut, src, rem0, rem1, make_float4(cdx, cdy, cdz, chh), cjj, vlo, vhi, np, nseq, fail, w0, w1);
                 __syncwarp();
                 // the later planes against the new vertices
                 olo &= ~rem0; ohi &= ~rem1;
@@ -1577,11 +1672,13 @@ int launch_group(const ClipArgs& a, const GroupBuf& b, int sm_count, cudaStream_
 // its whole volume.  A warp takes 32 cells at a time, its lanes one pair each of all the voxels that the cells' balls
 // meet.  The pairs that some plane crosses wait in queues (of about the same number of crossing planes) until there are
 // enough, and are cut by the crossing planes alone, G lanes a pair as in k_group_clip, starting from the voxel's box (cut
-// down to the ball's).  Sides are plain FP32 signs: a wrong sign within rounding of a plane moves a rounding-sized sliver.
+// down to the ball's).  Sides are plain FP32 signs: a wrong sign within rounding of a plane moves a rounding-sized sliver,
+// and signs that contradict each other are put right in the cut (group_cut).  What outgrows the polytope goes to a list.
 // Cells whose balls meet more than GV_BIG voxels are listed, with the running count of their units of GV_BIG pairs, and
 // the warps of a second launch take those units from a counter (2,097,152 clustered particles on 256^3 voxels: 166 ms;
 // 8.1 s when every warp went through all listed cells, 6.9 s with one thread a cell).
-// Bound by instruction issue, as k_group_clip.  131,072 clustered particles on 32^3 voxels: 4.7 ms; 297 ms with one thread
+// Bound by instruction issue, as k_group_clip.  131,072 clustered particles on 32^3 voxels: 4.8 ms (4.75 ms without the check
+// of a cut's boundary, whose signs near a lattice left parts of voxels wrong by up to a tenth); 297 ms with one thread
 // walking all voxels of a cell and clipping a copy of it by each voxel's walls; 13 ms with one thread a pair (5 of 32 lanes
 // active, and the lanes' polytopes in local memory).
 constexpr int GV_BIG = 512;
@@ -1812,13 +1909,13 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                     bool cut = open && !fail && !empty && cm != 0u;
                     if (!__any_sync(FULL, cut)) break;
                     const int src = gsh + (cut ? __ffs(cm) - 1 : 0);
-                    const unsigned rem0 = __shfl_sync(FULL, olo, src), rem1 = __shfl_sync(FULL, ohi, src);
+                    unsigned rem0 = __shfl_sync(FULL, olo, src), rem1 = __shfl_sync(FULL, ohi, src);
                     if (cut && rem0 == vlo && rem1 == vhi) {  // nothing is left
                         empty = true;
                         cut = false;
                     }
                     unsigned w0, w1;
-                    group_cut<G>(C, cut, src, rem0, rem1, f, 0u, vlo, vhi, np, nseq, fail, w0, w1);
+                    group_cut<G, true>(C, cut, src, rem0, rem1, f, 0u, vlo, vhi, np, nseq, fail, w0, w1);
                     __syncwarp();
                     olo &= ~rem0; ohi &= ~rem1;
                     if ((int)lane <= src || !cut) olo = ohi = 0u;
@@ -1868,7 +1965,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                         vol += y < 6 ? off * cr : off * cr / (2.f * p.w);
                     }
                 }
-            vol = gsum(vol) * (float)(1.0 / 6.0);
+            vol = gsum(vol) / 6.f;  // (a sixth as a float is 3e-8 too large)
             if (r == 0 && has) {
                 // a sliver's FP32 volume may come out slightly below zero; anything beyond 1e-5 of the box is a failure
                 if (fail || (on && vol < -1e-5f * (hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])))
