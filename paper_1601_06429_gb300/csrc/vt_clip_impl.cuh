@@ -954,7 +954,9 @@ __device__ __forceinline__ float trunc32(double v) {
 // A bisector with p cuts a vertex v off only when p lies in the ball around v through the site: whether the box [x0, x1]
 // x ... (relative to the site) reaches into the ball of any vertex of the cell, i.e. |v|^2 - |p - v|^2 >= -tol for some
 // v and p (balls widened by the vertices' error bounds).  Far sharper than the support of the cell's box where many
-// points lie just beyond the cell, at two dozen evaluations.
+// points lie just beyond the cell, at two dozen evaluations.  The FP32 rounding of the two squares is at most 13 u |v|^2 for
+// |p| < |v| (tol holds it for wider ones), which tol, on the scale of |v| times the search radius, falls below once
+// a vertex is some 70 radii away: FP32 vertices have it in their ev >= 8u |v|, FP64 ones need the term 2e-6 |v|^2.
 template <typename CT, int TP>
 __device__ __noinline__ bool ball_reaches(const WarpSmem<CT, TP>& S, float x0, float y0, float z0, float x1, float y1,
                                           float z1, float tol) {
@@ -968,8 +970,9 @@ __device__ __noinline__ bool ball_reaches(const WarpSmem<CT, TP>& S, float x0, f
             const float vx = trunc32(v.x), vy = trunc32(v.y), vz = trunc32(v.z), ev = trunc32(v.ev);
             const float dx = fmaxf(fmaxf(x0 - vx, vx - x1), 0.f), dy = fmaxf(fmaxf(y0 - vy, vy - y1), 0.f),
                         dz = fmaxf(fmaxf(z0 - vz, vz - z1), 0.f);
-            const float b = (vx * vx + vy * vy + vz * vz) - (dx * dx + dy * dy + dz * dz) +
-                            4.f * ev * (fabsf(vx) + fabsf(vy) + fabsf(vz) + ev);
+            const float v2 = vx * vx + vy * vy + vz * vz;
+            float b = v2 - (dx * dx + dy * dy + dz * dz) + 4.f * ev * (fabsf(vx) + fabsf(vy) + fabsf(vz) + ev);
+            if (sizeof(CT) == 8) b = fmaf(2e-6f, v2, b);
             best = fmaxf(best, b);
         }
     }
