@@ -73,7 +73,7 @@ typedef struct vt_params {
     int max_passes; /* candidate radius passes per cell before VT_ERR_SECURITY (default 1000) */
     int face_pool;  /* facet records reserved per particle (default 24; grown on demand) */
     int threads_per_cell; /* VT_FILTER32 only: 0 = the library's choice (default): 4 from 65,536 particles on (32
-                             where the device has no room for their memory), else 32; 32 = one warp per cell; 4 or
+                             where the device has no room for their memory, also later), else 32; 32 = one warp per cell; 4 or
                              8 = that many lanes per cell (8 or 4 cells per warp); 1 = one thread per cell, 32 cells
                              of a search-tree bucket per warp; but for 32, the cells the first kernels cannot finish
                              are then taken by a warp each (same cells; 4, 8 and 32 give the same bits).  4 and 8
@@ -390,9 +390,11 @@ int vt_last_error_detail(int *particle);
 
 /*
  * vt_debug_fail_alloc -- fault injection for tests (no counterpart in the paper): the nth device allocation
- * that vt_build or vt_build_batched makes for a handle's workspace from now on (counting from 1) fails as if
- * cudaMalloc had run out of memory, and the call returns VT_ERR_OOM after freeing what it had allocated (where the
- * library chose lane groups by itself, a failure of their memory makes it build with a warp per cell instead).  The
+ * for a handle's workspace from now on (counting from 1; vt_build, vt_build_owned and vt_build_batched, the growth of
+ * their facet pool, and what a handle's first calls of its products add) fails as if cudaMalloc had run out of memory,
+ * and the call returns VT_ERR_OOM after freeing what it had allocated (where the library chose lane groups by itself,
+ * their memory gives way: a failure of it, or of a later allocation, makes a warp take each cell instead, unless a
+ * captured vt_rebuild uses it).  The
  * hook fires once and disarms; nth <= 0 disarms it.  Process-wide (all host threads, all devices); returns the
  * previous setting (0 if the hook was disarmed or has fired).  Touches no device.
  */

@@ -257,6 +257,55 @@ GroupBuf group_buf(vt_handle h) {
     return b;
 }
 
+// the sets that take lane groups take a warp a cell instead
+__global__ void k_drop_group_modes(int32_t* set_cfg, int n) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n && ((set_cfg[k] >> 16) & 2)) set_cfg[k] &= 0xffff;
+}
+
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// Give the lane-group kernels' memory back; a warp takes each of their cells from now on (the same bits).
+void free_groups(vt_handle h) {
+    void* g[] = {h->spos4, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_act, h->g_ctr};
+    for (void* p : g)
+        if (p) pool_free(p, h->stream);
+    h->spos4 = nullptr;
+    h->g_stat = nullptr;
+    h->g_hdr = nullptr;
+    h->g_list = nullptr;
+    h->g_state = nullptr;
+    h->g_act = nullptr;
+    h->g_ctr = nullptr;
+    h->modes = (h->modes & ~12) | 1;
+    if (h->prm.threads_per_cell == 4 || h->prm.threads_per_cell == 8) h->prm.threads_per_cell = 32;
+}
+
+// An allocation after the handle's first ones, which stand beside the lane-group kernels' memory: where it fails, and
+// no one asked for lane groups by name, it takes their place.
+void* late_alloc(vt_handle h, size_t bytes) {
+    cudaStream_t s = h->stream;
+    void* p = injected_failure() ? nullptr : pool_alloc(bytes, s);
+    if (p || !h->g_state || !h->may_drop || h->captured || capturing(s)) return p;
+    if (h->set_cfg) {
+        k_drop_group_modes<<<(h->n_sets + 255) / 256, 256, 0, s>>>(h->set_cfg, h->n_sets);
+        h->n_launches += 1;
+    }
+    free_groups(h);
+    cudaStreamSynchronize(s);
+    cudaMemPool_t pool = device_pool();
+    if (pool) cudaMemPoolTrimTo(pool, 0);  // what they held can serve as one block
+    cudaGetLastError();
+    return pool_alloc(bytes, s);
+}
+
 int run_clip(vt_handle h) {
     cudaStream_t s = h->stream;
     for (int attempt = 0; attempt < 4; attempt++) {
@@ -283,7 +332,7 @@ int run_clip(vt_handle h) {
         uint64_t cap = h->face_cap * 2 > need ? h->face_cap * 2 : need;
         if (cap > 0xF0000000ull) return VT_ERR_CAPACITY;
         pool_free(h->faces, s);
-        h->faces = (Face*)pool_alloc(cap * sizeof(Face), s);
+        h->faces = (Face*)late_alloc(h, cap * sizeof(Face));
         if (!h->faces) return VT_ERR_OOM;
         h->face_cap = cap;
         h->hstat.error = 0;
@@ -399,6 +448,7 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
     h->prm = prm;
     h->geo = geo;
     h->n_sets = n_sets;
+    h->may_drop = chosen;
     h->stream = (cudaStream_t)stream;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -460,7 +510,7 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
             A.failed = true;
         }
     if (!A.failed && (h->modes & 12)) {
-        // last, so that what fits without the lane-group kernels' memory still fits
+        // last, and it gives way to later allocations (late_alloc): what fits without it still fits
         const size_t m = group_chunk(N);
         if (dtype == VT_F64) h->spos4 = A.get<float4>(N);
         h->g_stat = A.get<uint8_t>(m);
@@ -470,19 +520,9 @@ int build_impl(vt_handle* out, const void* pos, int dtype, const void* mass, int
         h->g_act = A.get<uint32_t>(2 * m);
         h->g_ctr = A.get<uint32_t>(group_counters(N));
         if (A.failed && chosen) {
-            void* g[] = {h->spos4, h->g_stat, h->g_hdr, h->g_list, h->g_state, h->g_act, h->g_ctr};
-            for (void* p : g)
-                if (p) pool_free(p, h->stream);
-            h->spos4 = nullptr;
-            h->g_stat = nullptr;
-            h->g_hdr = nullptr;
-            h->g_list = nullptr;
-            h->g_state = nullptr;
-            h->g_act = nullptr;
-            h->g_ctr = nullptr;
-            h->modes = 1;
-            h->prm.threads_per_cell = 32;
-            for (int k = 0; cfg_host && k < n_sets; k++) cfg_host[k] &= 0xffff;
+            free_groups(h);
+            for (int k = 0; cfg_host && k < n_sets; k++)
+                if ((cfg_host[k] >> 16) & 2) cfg_host[k] &= 0xffff;
             A.failed = false;
         }
     }
@@ -714,6 +754,7 @@ int vt_autotune_batched(const void* pos, int dtype, const int64_t* set_off, int 
 int vt_rebuild(vt_handle h, const void* pos, const void* mass) {
     if (!h || !pos) return VT_ERR_INVALID;
     cudaStream_t s = h->stream;
+    if (capturing(s)) h->captured = 1;
     // every counter, the work queues and the sticky error start at zero
     int rc = cuda_rc(cudaMemsetAsync(h->dstat, 0, sizeof(DevStatus), s));
     if (rc) return rc;
@@ -746,7 +787,7 @@ int vt_cells(vt_handle h, void* vol, int64_t* nbr_off, int32_t* nbr_id, int64_t*
         int64_t* off = nbr_off;
         if (!off) {
             if (!h->nbr_off_cache) {
-                h->nbr_off_cache = (int64_t*)pool_alloc((h->N + 1) * sizeof(int64_t), s);
+                h->nbr_off_cache = (int64_t*)late_alloc(h, (h->N + 1) * sizeof(int64_t));
                 if (!h->nbr_off_cache) return VT_ERR_OOM;
             }
             off = h->nbr_off_cache;
@@ -811,8 +852,8 @@ int vt_grid_density(vt_handle h, int G, int S, void* grid) {
 namespace {
 int ensure_retry(vt_handle h) {
     if (h->gretry) return VT_OK;
-    h->gretry = (int4*)pool_alloc((size_t)GRID_RETRY_CAP * sizeof(int4), h->stream);
-    h->gcnt = (unsigned*)pool_alloc(16 * sizeof(unsigned), h->stream);
+    if (!h->gcnt) h->gcnt = (unsigned*)late_alloc(h, 16 * sizeof(unsigned));
+    h->gretry = (int4*)late_alloc(h, (size_t)GRID_RETRY_CAP * sizeof(int4));
     if (!h->gretry || !h->gcnt) return VT_ERR_OOM;
     return VT_OK;
 }
@@ -837,7 +878,7 @@ int vt_grid_density_volume(vt_handle h, int G, void* grid) {
     if (h->gacc_n < n) {
         pool_free(h->gacc, h->stream);
         h->gacc_n = 0;
-        h->gacc = (double*)pool_alloc(n * sizeof(double), h->stream);
+        h->gacc = (double*)late_alloc(h, n * sizeof(double));
         if (!h->gacc) return VT_ERR_OOM;
         h->gacc_n = n;
     }

@@ -129,7 +129,9 @@ struct vt_handle_s {
     // exact workspace (per warp of the exact kernel)
     double* xws;
     int xws_warps;
-    // the lane-group kernels' memory (modes that use them only)
+    // the lane-group kernels' memory (modes that use them only); may_drop: no caller asked for them by name, so that they can be
+    // given up for a warp a cell; captured: a stream capture may hold their addresses
+    int may_drop, captured;
     uint8_t* g_stat;
     void* g_hdr;
     uint32_t* g_list;
