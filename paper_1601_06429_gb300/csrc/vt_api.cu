@@ -638,9 +638,9 @@ int vt_build_batched(vt_handle* out, const void* pos, int dtype, const void* mas
         // the thread-per-cell and lane-group kernels exist for the FP32 filter only
         cfg[k] = kt | (prm.precision == VT_FILTER32 && tpc_mode_of(tpc) > 0 ? tpc_mode_of(tpc) << 16 : 0);
     }
-    // the library's choice: no set asks for lane groups or one thread itself
-    bool chosen = !p || !p->threads_per_cell || p->threads_per_cell == 32;
-    for (int k = 0; set_tpc && k < n_sets; k++) chosen = chosen && (set_tpc[k] == 0 || set_tpc[k] == 32);
+    // the library's choice: no one asks for lane groups by name, neither p for all sets nor set_tpc, which replaces p's, for one
+    bool chosen = set_tpc || !p || (p->threads_per_cell != 4 && p->threads_per_cell != 8);
+    for (int k = 0; set_tpc && k < n_sets; k++) chosen = chosen && set_tpc[k] != 4 && set_tpc[k] != 8;
     if (!rc) rc = build_impl(out, pos, dtype, mass, N, sg[0], n_sets, set_off, sg, cfg, prm, chosen, stream);
     delete[] sg;
     delete[] cfg;

@@ -90,3 +90,30 @@ def test_a_captured_rebuild_keeps_its_memory():
     g.replay()
     torch.cuda.synchronize()
     assert vt.vt_status(h)["rc"] == 0 and same(h, ref)
+
+
+@pytest.mark.parametrize("tpc,set_tpc,falls_back", [
+    (4, 0, True), (4, None, False), (0, None, True), (0, 4, False), (32, (1, 0), True), (0, (1, 8), False)])
+def test_whose_choice_lane_groups_of_a_batch_are(tpc, set_tpc, falls_back):
+    """The last allocation of a batch that takes lane groups is theirs: set_tpc (0: the library's choice), where it is
+    given, replaces threads_per_cell."""
+    n = 2
+    off = np.array([0, N // 2, N + 1000], np.int64)
+    pos = torch.from_numpy(inputs.uniform(int(off[-1]), seed=7, dtype=np.float32)).cuda()
+    boxes = np.tile([0.0, 0.0, 0.0, 1.0, 1.0, 1.0], (n, 1))
+    kw = {"threads_per_cell": tpc}
+    if set_tpc is not None:
+        kw["set_tpc"] = np.broadcast_to(np.array(set_tpc, np.int32), (n,)).copy()
+    vol = vt.cells(vt.vt_build_batched(pos, off, boxes, **kw))[0]
+    vt.vt_debug_fail_alloc(1000)
+    vt.vt_destroy(vt.vt_build_batched(pos, off, boxes, **kw))
+    last = 1000 - vt.vt_debug_fail_alloc(0)
+    vt.vt_debug_fail_alloc(last)
+    if falls_back:
+        h = vt.vt_build_batched(pos, off, boxes, **kw)
+        assert vt.vt_debug_fail_alloc(0) == 0
+        assert torch.equal(vt.cells(h)[0], vol)
+    else:
+        with pytest.raises(vt.VTError) as e:
+            vt.vt_build_batched(pos, off, boxes, **kw)
+        assert e.value.code == vt.VT_ERR_OOM
