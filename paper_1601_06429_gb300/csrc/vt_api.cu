@@ -852,7 +852,7 @@ int vt_grid_density(vt_handle h, int G, int S, void* grid) {
 namespace {
 int ensure_retry(vt_handle h) {
     if (h->gretry) return VT_OK;
-    if (!h->gcnt) h->gcnt = (unsigned*)late_alloc(h, 16 * sizeof(unsigned));
+    if (!h->gcnt) h->gcnt = (GridCounters*)late_alloc(h, sizeof(GridCounters));
     h->gretry = (int4*)late_alloc(h, (size_t)GRID_RETRY_CAP * sizeof(int4));
     if (!h->gretry || !h->gcnt) return VT_ERR_OOM;
     return VT_OK;
@@ -930,8 +930,8 @@ int vt_status(vt_handle h, vt_stats* out) {
     out->reserved[2] = (int64_t)d.n_collected;
     out->n_handed_over = h->n_owned < h->N ? 0 : (int64_t)d.n_warp_cells;
     if (h->gcnt) {
-        unsigned gc[2] = {0u, 0u};
-        if (cudaMemcpy(gc, h->gcnt, sizeof(gc), cudaMemcpyDeviceToHost) == cudaSuccess) out->n_grid_failed = gc[1];
+        unsigned failed = 0u;
+        if (cudaMemcpy(&failed, &h->gcnt->n_fail, sizeof(failed), cudaMemcpyDeviceToHost) == cudaSuccess) out->n_grid_failed = failed;
         else cudaGetLastError();
     }
     out->n_bucket_passes = (int64_t)d.n_bucket_passes;

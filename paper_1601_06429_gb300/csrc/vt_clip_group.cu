@@ -1703,7 +1703,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
     GCell& C = cells[gsh / G];
     const P* const spos = (const P*)A.spos;
     const double vox = A.h[0] * A.h[1] * A.h[2];
-    const unsigned long long listed = BIG ? *((volatile unsigned long long*)A.n_big) : 0ull;
+    const unsigned long long listed = BIG ? *((volatile unsigned long long*)&A.ctr->n_big) : 0ull;
     const unsigned long long n_units = listed & ((1ull << BIG_BITS) - 1ull);
     auto gballot = [&](bool p) -> unsigned { return (__ballot_sync(FULL, p) >> gsh) & GM; };
     auto gsum = [&](float v) -> float {
@@ -1725,7 +1725,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
             if (BIG) {
                 // one unit of a listed cell: the last cell whose first unit is not beyond it
                 unsigned long long u = 0;
-                if (lane == 0) u = atomicAdd(A.big_queue, 1ull);
+                if (lane == 0) u = atomicAdd(&A.ctr->big_queue, 1ull);
                 u = __shfl_sync(FULL, u, 0);
                 if (u >= n_units) more = false;
                 else {
@@ -1749,7 +1749,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                     total = min(total, t1 + GV_BIG);
                 }
             } else {
-                if (lane == 0) b = atomicAdd(A.queue, 32u);
+                if (lane == 0) b = atomicAdd(&A.ctr->queue, 32u);
                 b = __shfl_sync(FULL, b, 0);
                 if ((int64_t)b >= A.N) more = false;
                 else {
@@ -1769,7 +1769,7 @@ __global__ void __launch_bounds__(32, 9) k_group_voxels(const __grid_constant__ 
                             atomicAdd(&A.acc[(v[2] * A.G + v[1]) * A.G + v[0]], A.dens[k] * A.cell[k].vol);
                         } else if (mm > GV_BIG) {
                             const unsigned long long o =
-                                atomicAdd(A.n_big, (1ull << BIG_BITS) + (unsigned long long)((mm + GV_BIG - 1) / GV_BIG));
+                                atomicAdd(&A.ctr->n_big, (1ull << BIG_BITS) + (unsigned long long)((mm + GV_BIG - 1) / GV_BIG));
                             A.big[o >> BIG_BITS] = (uint32_t)k;
                             A.big_unit[o >> BIG_BITS] = o & ((1ull << BIG_BITS) - 1ull);
                         } else {

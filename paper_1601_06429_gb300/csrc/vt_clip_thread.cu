@@ -913,7 +913,7 @@ template <typename P>
 __global__ void __launch_bounds__(32) k_grid_volume(GridArgs A) {
     __shared__ Poly<256, 130> C;
     if (threadIdx.x) return;
-    const int64_t n = (int64_t)min(*((volatile unsigned*)A.n_retry), A.retry_cap);
+    const int64_t n = (int64_t)min(*((volatile unsigned*)&A.ctr->n_retry), A.retry_cap);
     for (int64_t e = blockIdx.x; e < n; e += gridDim.x) {
         const int4 ent = A.retry[e];
         const int64_t k = (int64_t)ent.x;
@@ -932,7 +932,7 @@ __global__ void __launch_bounds__(32) k_grid_volume(GridArgs A) {
             if (fmaxf(f.x * lo[0], f.x * hi[0]) + fmaxf(f.y * lo[1], f.y * hi[1]) + fmaxf(f.z * lo[2], f.z * hi[2]) > f.w)
                 r = C.cut(f);
         }
-        if (r < 0) grid_fail(A, TF_CAP);
+        if (r < 0) grid_fail(A);
         if (r) continue;
         const float vol = C.volume();
         if (vol > 0.f) atomicAdd(&A.acc[vi], A.dens[k] * (double)vol);
@@ -971,8 +971,7 @@ struct CvtArgs {
     void* out;            // dE_w / dx, input order [N][3]
     int4* retry;
     unsigned retry_cap;
-    unsigned* n_retry;
-    unsigned* n_fail;
+    GridCounters* ctr;
 };
 
 // dE_w/dx_k = 2 w_k V_k (x_k - z_k) + sum over facets (w_k - w_j) / |d| integral_f |y - x_k|^2 (y - x_k) dA.
@@ -1112,9 +1111,9 @@ __global__ void __launch_bounds__(128) k_cvt_facets(CvtArgs A) {
     }
     if (r != 0 || !in) return;
     if (fail) {
-        const unsigned slot = atomicAdd(A.n_retry, 1u);
+        const unsigned slot = atomicAdd(&A.ctr->n_retry, 1u);
         if (slot < A.retry_cap) A.retry[slot] = make_int4((int)k, 0, 0, 0);
-        else atomicAdd(A.n_fail, 1u);
+        else atomicAdd(&A.ctr->n_fail, 1u);
         return;
     }
     const CellOut co = A.cell[k];
@@ -1133,7 +1132,7 @@ __global__ void __launch_bounds__(128) k_cvt_facets(CvtArgs A) {
 // ordered by angle in the facet plane and fanned.
 template <typename P, class CL>
 __global__ void __launch_bounds__(128) k_cvt_weighted(CvtArgs A) {
-    const int64_t n = (int64_t)min(*((volatile unsigned*)A.n_retry), A.retry_cap);
+    const int64_t n = (int64_t)min(*((volatile unsigned*)&A.ctr->n_retry), A.retry_cap);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = (int64_t)A.retry[e].x;
         const P pi = ((const P*)A.spos)[k];
@@ -1142,7 +1141,7 @@ __global__ void __launch_bounds__(128) k_cvt_weighted(CvtArgs A) {
         CL C;
         const int f = grid_cell<P, CL>(C, ga, k, pi);
         if (f) {
-            atomicAdd(A.n_fail, 1u);
+            atomicAdd(&A.ctr->n_fail, 1u);
             continue;
         }
         const uint32_t ik = A.perm[k];
@@ -1226,20 +1225,17 @@ __global__ void k_grid_finish(const double* __restrict__ acc, int64_t n, double 
 
 int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
                        const uint32_t* face_start, const uint16_t* face_count, const double* dens_sorted, const float* rad,
-                       const CellOut* cell, uint32_t* big, uint64_t* big_unit, int G, double* acc, int4* retry, unsigned retry_cap, unsigned* counters, void* out, int sm_count,
+                       const CellOut* cell, uint32_t* big, uint64_t* big_unit, int G, double* acc, int4* retry, unsigned retry_cap, GridCounters* counters, void* out, int sm_count,
                        cudaStream_t s) {
     GridArgs a;
     a.spos = spos; a.N = N; a.geo = g; a.faces = faces; a.face_start = face_start; a.face_count = face_count;
     a.dens = dens_sorted; a.G = G; a.acc = acc; a.retry = retry; a.retry_cap = retry_cap;
-    a.n_retry = counters; a.n_fail = counters + 1;
+    a.ctr = counters;
     for (int c = 0; c < 3; c++) a.h[c] = g.L[c] / G;
     const int64_t n = (int64_t)G * G * G;
     cudaMemsetAsync(acc, 0, n * sizeof(double), s);
-    cudaMemsetAsync(counters, 0, 16 * sizeof(unsigned), s);
+    cudaMemsetAsync(counters, 0, sizeof(GridCounters), s);
     a.rad = rad; a.cell = cell; a.big = big; a.big_unit = big_unit;
-    a.queue = counters + 2;
-    a.n_big = reinterpret_cast<unsigned long long*>(counters + 4);
-    a.big_queue = reinterpret_cast<unsigned long long*>(counters + 6);
     launch_grid_pairs(a, dtype, sm_count, s);
     const unsigned rb = (unsigned)(sm_count * 16);
     if (dtype == VT_F32) k_grid_volume<float4><<<rb, 32, 0, s>>>(a);
@@ -1254,12 +1250,12 @@ int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g
 int launch_cvt_weighted(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
                         const uint32_t* face_start, const uint16_t* face_count, const CellOut* cell, const float* rad,
                         const uint32_t* perm, const void* w, void* out, int4* retry, unsigned retry_cap,
-                        unsigned* counters, int sm_count, cudaStream_t s) {
+                        GridCounters* counters, int sm_count, cudaStream_t s) {
     CvtArgs a;
     a.spos = spos; a.N = N; a.geo = g; a.faces = faces; a.face_start = face_start; a.face_count = face_count;
     a.cell = cell; a.rad = rad; a.perm = perm; a.w = w; a.dtype = dtype; a.out = out; a.retry = retry; a.retry_cap = retry_cap;
-    a.n_retry = counters; a.n_fail = counters + 1;
-    cudaMemsetAsync(counters, 0, 16 * sizeof(unsigned), s);
+    a.ctr = counters;
+    cudaMemsetAsync(counters, 0, sizeof(GridCounters), s);
     const unsigned nb = (unsigned)((N + 128 / CVT_LANES - 1) / (128 / CVT_LANES));
     const unsigned rb = (unsigned)(sm_count * 4);
     if (dtype == VT_F32) {

@@ -16,28 +16,21 @@ struct GridArgs {
     const CellOut* cell;
     uint32_t* big;       // cells whose ball meets more than GV_BIG voxels, and the first unit of work of each
     uint64_t* big_unit;
-    unsigned long long* n_big;  // listed cells above bit BIG_BITS, their units of GV_BIG pairs below
-    unsigned long long* big_queue;
-    unsigned* queue;
+    GridCounters* ctr;
     int G;
     double h[3];         // voxel side L / G
     double* acc;         // [G^3] sum of rho |cell & voxel|
-    int4* retry;         // (cell, voxel x, y, z unwrapped) for the larger cell type
+    int4* retry;         // (cell, voxel x, y, z unwrapped) for the larger polytope
     unsigned retry_cap;
-    unsigned* n_retry;
-    unsigned* n_fail;
 };
 
-// a part that cannot be computed: counted in total and by reason (counters[4 + code])
-__device__ __forceinline__ void grid_fail(const GridArgs& A, int code) {
-    atomicAdd(A.n_fail, 1u);
-    atomicAdd(A.n_fail + 3 + (code > 0 && code < 12 ? code : 0), 1u);
-}
+// a part that cannot be computed
+__device__ __forceinline__ void grid_fail(const GridArgs& A) { atomicAdd(&A.ctr->n_fail, 1u); }
 
 __device__ __forceinline__ void push_retry(const GridArgs& A, int64_t k, int ax, int ay, int az) {
-    const unsigned slot = atomicAdd(A.n_retry, 1u);
+    const unsigned slot = atomicAdd(&A.ctr->n_retry, 1u);
     if (slot < A.retry_cap) A.retry[slot] = make_int4((int)k, ax, ay, az);
-    else grid_fail(A, 11);
+    else grid_fail(A);
 }
 
 // the voxels that the ball of sorted particle k meets: first index and count per axis; returns their number

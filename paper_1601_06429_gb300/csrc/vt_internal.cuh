@@ -7,6 +7,8 @@
 
 namespace vt {
 
+struct GridCounters;  // vt_kernels.cuh
+
 constexpr int WARP = 32;
 constexpr int STACK_CAP = 192;  // tree traversal stack per warp (fast clipping kernels)
 constexpr int MAX_FACETS = 510; // facets of one cell (the exact kernel's plane capacity minus the initial six)
@@ -148,11 +150,11 @@ struct vt_handle_s {
     vt::DevStatus* smap;    // mapped pinned host block through which the status words are read
     int64_t n_faces;
     int faces_on_device;    // set by vt_rebuild: the facet count is read from the device from then on
-    // volume-averaged grid: accumulator, retry list of the larger cell type, counters (retries, failures)
+    // volume-averaged grid: accumulator, list of the pairs for the larger polytope, counters
     double* gacc;
     int64_t gacc_n;
     int4* gretry;
-    unsigned* gcnt;         // [16]: retries, failures, -, by reason (4 + code)
+    vt::GridCounters* gcnt;
     int sm_count;
     int64_t n_launches;
     double t_sort_ms, t_clip_ms;

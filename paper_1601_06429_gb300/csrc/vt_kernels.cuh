@@ -109,16 +109,24 @@ int launch_clip(const ClipArgs& a, const GroupBuf* gb, int dtype, int precision,
 int launch_clip_exact(const ClipArgs& a, int dtype, int sm_count, cudaStream_t s);
 int launch_clip_thread(const ClipArgs& a, int dtype, int sm_count, cudaStream_t s);
 int launch_clip_group(const ClipArgs& a, const GroupBuf& b, int dtype, int lanes, int sm_count, cudaStream_t s);
+// Counters of the volume-averaged grid and of the weighted gradient, zero before their launches
+struct GridCounters {
+    unsigned n_retry, n_fail;  // listed pairs (cells), parts that could not be computed
+    unsigned queue;            // next cells to look at
+    unsigned pad;
+    unsigned long long n_big;      // listed cells over many voxels above bit BIG_BITS, their units of GV_BIG pairs below
+    unsigned long long big_queue;  // next unit
+};
 int launch_fma_probe(int blocks, int iters, float* sink, cudaStream_t s);
 int launch_fma_probe64(int blocks, int iters, double* sink, cudaStream_t s);
 int launch_cvt_weighted(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
                         const uint32_t* face_start, const uint16_t* face_count, const CellOut* cell, const float* rad,
                         const uint32_t* perm, const void* w, void* out, int4* retry, unsigned retry_cap,
-                        unsigned* counters, int sm_count, cudaStream_t s);
+                        GridCounters* counters, int sm_count, cudaStream_t s);
 int launch_grid_volume(const void* spos, int dtype, int64_t N, const Geometry& g, const Face* faces,
                        const uint32_t* face_start, const uint16_t* face_count, const double* dens_sorted, const float* rad,
                        const CellOut* cell, uint32_t* big, uint64_t* big_unit, int G, double* acc, int4* retry, unsigned retry_cap,
-                       unsigned* counters, void* out, int sm_count,
+                       GridCounters* counters, void* out, int sm_count,
                        cudaStream_t s);
 int launch_gradient_gg(const Face* faces, const uint32_t* face_start, const uint16_t* face_count, const CellOut* cell,
                        const double* dens_sorted, const uint32_t* perm, int64_t N, void* grad, int dtype,

@@ -54,13 +54,28 @@ def test_lattices_close_to_degenerate(kind, shift, G, oracle_mod):
     check(lattice(kind, shift, seed=G), G, True, "plain64", oracle_mod)
 
 
-@pytest.mark.parametrize("facets", [30, 60, 110])
-@pytest.mark.parametrize("G", [2, 3, 7])
-def test_cells_of_many_facets(facets, G, oracle_mod):
-    """A particle inside a sphere of others: at G = 3 the middle voxel takes nearly all of its facets."""
+def sphere(facets):
+    """A particle inside a sphere of others, whose cell has that many facets."""
     g = inputs.rng(facets)
     k = np.arange(facets)
     z, phi = 1.0 - (2.0 * k + 1.0) / facets, k * (np.pi * (3.0 - np.sqrt(5.0)))
     s = np.stack([np.sqrt(1.0 - z * z) * np.cos(phi), np.sqrt(1.0 - z * z) * np.sin(phi), z], 1)
-    x = np.concatenate([[[0.5, 0.5, 0.5]], 0.5 + (0.36 + 1e-4 * g.random((facets, 1))) * s]).astype(np.float32)
-    check(x, G, False, "filter32", oracle_mod)
+    return np.concatenate([[[0.5, 0.5, 0.5]], 0.5 + (0.36 + 1e-4 * g.random((facets, 1))) * s]).astype(np.float32)
+
+
+@pytest.mark.parametrize("facets", [30, 60, 110])
+@pytest.mark.parametrize("G", [2, 3, 7])
+def test_cells_of_many_facets(facets, G, oracle_mod):
+    """At G = 3 the middle voxel takes nearly all of the facets."""
+    check(sphere(facets), G, False, "filter32", oracle_mod)
+
+
+def test_parts_beyond_the_larger_polytope_are_counted():
+    """260 facets, of which the middle voxel of 3 holds some 200 (130 fit); the same handle then fills 7^3 voxels."""
+    x = sphere(260)
+    h = vt.vt_build(torch.from_numpy(x).cuda(), None, (0.0,) * 3, (1.0,) * 3, False)
+    vt.grid_density_volume(h, 3)
+    assert vt.vt_status(h)["n_grid_failed"] == 1
+    got = vt.grid_density_volume(h, 7).double()
+    assert vt.vt_status(h)["n_grid_failed"] == 0
+    assert abs(float(got.mean()) - len(x)) <= 1e-5 * len(x)  # every particle has mass 1
