@@ -71,8 +71,8 @@ def test_cells_of_many_facets(facets, G, oracle_mod):
 
 
 def test_parts_beyond_the_larger_polytope_are_counted():
-    """260 facets, of which the middle voxel of 3 holds some 200 (130 fit); the same handle then fills 7^3 voxels."""
-    x = sphere(260)
+    """200 facets, of which the middle voxel of 3 holds some 150 (130 fit); the same handle then fills 7^3 voxels."""
+    x = sphere(200)
     h = vt.vt_build(torch.from_numpy(x).cuda(), None, (0.0,) * 3, (1.0,) * 3, False)
     vt.grid_density_volume(h, 3)
     assert vt.vt_status(h)["n_grid_failed"] == 1
