@@ -928,7 +928,8 @@ int vt_status(vt_handle h, vt_stats* out) {
     out->reserved[0] = d.error_detail;
     out->reserved[1] = (int64_t)d.n_collect;
     out->reserved[2] = (int64_t)d.n_collected;
-    out->n_handed_over = h->n_owned < h->N ? 0 : (int64_t)d.n_warp_cells;
+    // (a warp kernel that takes every cell, of a list in an owned build, gets none handed over)
+    out->n_handed_over = h->n_owned < h->N && (h->modes & ~1) == 0 ? 0 : (int64_t)d.n_warp_cells;
     if (h->gcnt) {
         unsigned failed = 0u;
         if (cudaMemcpy(&failed, &h->gcnt->n_fail, sizeof(failed), cudaMemcpyDeviceToHost) == cudaSuccess) out->n_grid_failed = failed;
