@@ -211,23 +211,53 @@ int launch_gradient(const Face* faces, const uint32_t* face_start, const uint16_
     return 1;
 }
 
-// a / |(x, y, z)| to 1e-13 (results in FP32 only: they are the same ones), in FP32 but for the last sum: the FP32 reciprocal root s, the residual e = 1 - d^2 s^2 of it
-// with d^2 and s^2 as unevaluated sums of two floats, and 1/|d| = s (1 + e/2 + 3/8 e^2) to third order in e < 1e-6
+// exact product and sum as a float and its remainder (Dekker, Knuth)
+__device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
+    p = __fmul_rn(a, b);
+    e = __fmaf_rn(a, b, -p);
+}
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+// a / |(x, y, z)| to 1.3 x 2^-53 (an FP64 root and quotient: 2.7 x), with two FP64 sums and the rest in FP32, 64 times the
+// rate: the reciprocal root s, the residual e = 1 - d^2 s^2 of it, |e| < 2^-21, with d^2 as the sum of three floats, s^2
+// of two, e of two, and a/|d| = a s (1 + e/2 + 3/8 e^2), the next term below 2^-64.
 __device__ __forceinline__ double over_dist(float a, float x, float y, float z) {
-    const float xx = x * x, yy = y * y, zz = z * z;
-    const float s1 = __fadd_rn(xx, yy), b1 = __fsub_rn(s1, xx);
-    const float d2 = __fadd_rn(s1, zz), b2 = __fsub_rn(d2, s1);
-    if (!(d2 > 1e-26f && d2 < 1e26f)) {  // outside, the low parts would leave the range of a float
+    float xx, xl, yy, yl, zz, zl, s1, dh, dm, e1, e2, m1, m2, f1, f2, f3, f4;
+    two_prod(x, x, xx, xl);
+    two_prod(y, y, yy, yl);
+    two_prod(z, z, zz, zl);
+    two_sum(xx, yy, s1, e1);
+    two_sum(s1, zz, dh, e2);
+    const float s = rsqrtf(dh);
+    float p, pr;
+    two_prod(a, s, p, pr);
+    if (!(dh > 1e-26f && dh < 1e26f && p > 1e-28f)) {  // outside, the low parts would leave the range of a float
         const double X = x, Y = y, Z = z;
         return (double)a / sqrt(fma(Z, Z, fma(Y, Y, X * X)));
     }
-    const float t1 = __fadd_rn(__fsub_rn(xx, __fsub_rn(s1, b1)), __fsub_rn(yy, b1));
-    const float t2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(d2, b2)), __fsub_rn(zz, b2));
-    const float lo = ((fmaf(x, x, -xx) + fmaf(y, y, -yy)) + fmaf(z, z, -zz)) + (t1 + t2);
-    const float s = rsqrtf(d2), ss = s * s, sl = fmaf(s, s, -ss);
-    const float e = fmaf(-lo, ss, fmaf(-d2, sl, fmaf(-d2, ss, 1.f)));
-    const float p = a * s;
-    return f2d(p) + f2d(fmaf(p, e * fmaf(0.375f, e, 0.5f), fmaf(a, s, -p)));
+    two_sum(e1, e2, m1, f1);
+    two_sum(m1, xl, m2, f2);
+    two_sum(m2, yl, m1, f3);
+    two_sum(m1, zl, dm, f4);
+    const float dl = (f1 + f2) + (f3 + f4);
+    float ss, sl, ph, pl, q1, q1l, q2, q2l;
+    two_prod(s, s, ss, sl);
+    two_prod(dh, ss, ph, pl);
+    two_prod(dh, sl, q1, q1l);
+    two_prod(dm, ss, q2, q2l);
+    float t1, t2, eh, r1, r2, r3;
+    two_sum(__fsub_rn(1.f, ph), -pl, t1, r1);
+    two_sum(t1, -q1, t2, r2);
+    two_sum(t2, -q2, eh, r3);
+    const float el = (r1 + r2) + (r3 - ((q1l + q2l) + fmaf(dm, sl, dl * ss)));
+    const float hh = 0.5f * eh, hl = fmaf(0.375f * eh, eh, 0.5f * el);
+    float th, tl, uh, ul;
+    two_prod(p, hh, th, tl);
+    two_sum(pr, th, uh, ul);
+    return f2d(p) + (f2d(uh) + f2d(ul + (tl + fmaf(p, hl, pr * hh))));
 }
 
 // ------------------------------------------------------------------ Green-Gauss gradient
@@ -235,9 +265,10 @@ __device__ __forceinline__ double over_dist(float a, float x, float y, float z) 
 // centroid relative to x_i and d_f the neighbour image's displacement: the surface integral of rho n over the
 // cell with rho at a facet centroid interpolated linearly between the two sites, exact for a linear field
 // (the tangential parts cancel on a closed Voronoi cell); on a box wall rho is taken as rho_i.  One thread per
-// cell, FP64 sums over FP32 facet records: six FP64 instructions a facet (FP32 results), and the gathers of records and
-// densities, bound it (one million clustered cells: 522 us; 1465 us with an FP64 root and quotient a facet).  FP64 results
-// keep the FP64 root and quotient.
+// cell, FP64 sums over FP32 facet records: seven FP64 instructions a facet (FP32 results), and the gathers of records and
+// densities, bound it (one million clustered cells: 625 us; 1465 us with an FP64 root and quotient a facet, 535 us with a
+// quotient to 1e-13 from pairs of floats, which changed the last bit of a result now and then).  FP64 results keep the FP64
+// root and quotient.
 template <typename T>
 __global__ void k_gradient_gg(const Face* __restrict__ faces, const uint32_t* __restrict__ face_start,
                               const uint16_t* __restrict__ face_count, const CellOut* __restrict__ cell,
