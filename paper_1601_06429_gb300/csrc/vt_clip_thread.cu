@@ -1091,7 +1091,8 @@ __global__ void __launch_bounds__(128) k_cvt_facets(CvtArgs A) {
                     const float wr = (g == 0 ? -27.f / 48.f : 25.f / 48.f) * (oo + s * s + tt * tt);
                     i0 += wr; is += wr * s; it += wr * tt;
                 }
-                m0 += (double)(at * i0); ms += (double)(at * is); mt += (double)(at * it);
+                const double ad = f2d(at);
+                m0 = fma(ad, f2d(i0), m0); ms = fma(ad, f2d(is), ms); mt = fma(ad, f2d(it), mt);
             }
             const uint32_t ij = A.perm[__float_as_uint(reinterpret_cast<const float4*>(&A.faces[st + q])[1].w)];
             const double wj = A.dtype == VT_F32 ? (double)((const float*)A.w)[ij] : ((const double*)A.w)[ij];

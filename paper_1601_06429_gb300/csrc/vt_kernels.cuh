@@ -12,6 +12,14 @@ struct __align__(32) dpt4 {
     double x, y, z, w;
 };
 
+// A float as a double by integer arithmetic (the conversion instruction runs at the FP64 rate, 1/64 of the FP32 one);
+// zeros and denormals, which the shift would misplace, and the rest take the same bits as a cast.
+__device__ __forceinline__ double f2d(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m < 0x00800000u || m >= 0x7f800000u) return (double)v;
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
 size_t scan_tmp_bytes(int64_t n);
 size_t radix_tmp_bytes(int64_t N);
 int scan_u32_u32(const uint32_t* in, uint32_t* out, int64_t n, void* tmp, cudaStream_t s);

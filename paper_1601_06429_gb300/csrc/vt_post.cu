@@ -153,13 +153,7 @@ int launch_nbr_emit(const Face* faces, const uint32_t* face_start, const uint16_
 }
 
 // Facet records are FP32 and the sums over them FP64, which runs at 1/64 of the FP32 rate: what bounds the gradient
-// kernels is the count of FP64 instructions.  A float as a double by integer arithmetic (the conversion instruction runs
-// at the FP64 rate too); zeros and denormals, which the shift would misplace, and the rest take the same bits as a cast.
-__device__ __forceinline__ double f2d(float v) {
-    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
-    if (m < 0x00800000u || m >= 0x7f800000u) return (double)v;
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-}
+// kernels is the count of FP64 instructions (f2d converts without one).
 
 // ------------------------------------------------------------------ density gradient
 // Implementation section ("density gradient ... using density and neighboring information"); reading:
