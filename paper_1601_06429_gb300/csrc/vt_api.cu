@@ -370,10 +370,11 @@ int vt_default_params(vt_params* p) {
 namespace {
 
 // Threads per cell where the caller leaves the choice to the library (0).  FP32 filter: 4 lanes a cell from 65,536
-// particles on, where the chip has enough cells for 8 of them to share a warp; clipping 40,000 / 65,536 / 100,000 /
-// 2,097,152 uniform points takes 1.98 / 3.18 / 4.95 / 114.5 ms by a warp a cell and 1.69 / 2.30 / 2.88 / 40.2 ms by 4
-// lanes, 65,537 / 100,000 / 200,000 / 2,097,152 clustered points 4.72 / 6.76 / 13.1 / 128 ms and 5.27 / 5.99 / 9.08 /
-// 61 ms (8 lanes are slower than 4 at every size).
+// particles on, where the chip has enough cells for 8 of them to share a warp.  Clip times by a warp a cell and by 4 lanes:
+// 40,000 / 65,536 / 100,000 / 2,097,152 uniform points 1.98 / 3.18 / 4.90 / 114.5 ms and 1.69 / 2.28 / 2.65 / 40.2 ms;
+// 65,536 / 75,000 / 85,000 / 100,000 / 200,000 / 2,097,152 clustered points 4.49 / 4.93 / 5.72 / 6.10 / 13.1 / 128 ms and 4.84 /
+// 5.07 / 5.33 / 5.82 / 9.08 / 61 ms.  Uniform points gain from fewer on and clustered ones from 80,000: the line lies
+// between (8 lanes are slower than 4 at every size).
 constexpr int64_t GROUP_MIN_N = 65536;
 int default_tpc(int precision, int64_t N) { return precision == VT_FILTER32 && N >= GROUP_MIN_N ? 4 : 32; }
 

@@ -1298,7 +1298,6 @@ __global__ void __launch_bounds__(32, G == 4 ? 11 : 20) k_group_clip(const __gri
 #pragma unroll 1
             for (int p = r; p < np; p += G) { K->Pl[p] = C.Pl[p]; K->Ps[p] = C.Ps[p]; K->Sq[p] = C.Sq[p]; }
             if (r == 0) {
-                H.R2 = R2;
                 H.bx0 = bx0; H.by0 = by0; H.bz0 = bz0; H.bx1 = bx1; H.by1 = by1; H.bz1 = bz1;
                 H.meta |= w64 << 16;
                 B.hdr[ci] = H;

@@ -84,15 +84,15 @@ struct ClipArgs {
     float* rad;
 };
 // The lane-group kernels' memory (vt_clip_group.cu): per cell of a chunk its status, header, candidate list and the
-// state kept between radius passes (2.2 KB a cell; chunks of at most GROUP_CHUNK cells), and the queue counters of
-// every launch.
+// state kept between radius passes (with the lists of cells 2.6 KB a cell; chunks of at most GROUP_CHUNK cells), and the
+// queue counters of every launch.
 constexpr int GROUP_CAND = 96;
 constexpr int GROUP_NT = 64, GROUP_NP = 40;  // vertex slots and planes of a cell
 constexpr int GROUP_STATE = (GROUP_NT * 20 + GROUP_NP * 21 + 15) / 16 * 16;
 constexpr int GROUP_PASSES = 12;
 constexpr uint32_t GROUP_CHUNK = 1u << 21;
-struct GHdr {
-    float rlo2, rhi2, B, R2, cap2;            // range of |d|^2 of the pass, start box, squared radius, widest search
+struct __align__(16) GHdr {
+    float rlo2, rhi2, B, cap2;                // range of |d|^2 of the pass, start box, widest search
     float bx0, by0, bz0, bx1, by1, bz1;       // box around the vertices
     uint32_t vlo, vhi, n, meta;               // slots in use; candidates | cuts so far << 16; planes | start walls << 8 | FP64 << 16 | passes << 24
     float first2;                             // squared first radius
