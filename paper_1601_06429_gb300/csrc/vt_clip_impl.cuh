@@ -51,10 +51,12 @@ struct Cap {
     static constexpr int CAND = 256;                      // candidates per radius pass
     static constexpr int STACK = TP <= 4 ? STACK_CAP : 4 * STACK_CAP;
 };
-// From this radius pass on (from the second one for listed cells) a search also tests nodes and points against the balls
-// of the cell's vertices: the cells that get there bound a void beside dense halos, and without it collect thousands of
-// halo points in passes of 256.
+// From this radius pass on (from the second one for listed cells) a search that overflows the candidate list also tests nodes
+// and points against the balls of the cell's vertices, and so do the cell's later ones: such a cell bounds a void beside
+// dense halos, and without it collects thousands of halo points in passes of 256.  Listed cells, nearly all of that kind, and
+// FP64 cells, whose candidates cost more, do it whether a search overflows or not.
 constexpr int BALL_PASS = 2;
+constexpr int BALL_FULL = 8;   // overflows of a cell's searches with the balls after which it is looked whether they help
 
 template <typename CT> struct Prec;
 template <> struct Prec<float> {
@@ -1335,12 +1337,22 @@ __device__ int do_cell(WarpSmem<CT, TP>& S, const ClipArgs& A, uint32_t self, do
                          : (CT)(4.0 * (g.L[0] * g.L[0] + g.L[1] * g.L[1] + g.L[2] * g.L[2]));
     bool done = false;
     bool need_exact = false, ovf = false;
+    // The balls cost two to five times the rest of a search.  FP32 cells that are not listed take them up at their first
+    // overflow (asked in every search they cost a sheet of 70,000 particles, 1e-2 of the box thick, 7.9 ms where 7.2 do; FP64
+    // cells gain by them without, 2 % for 30,011 clustered particles, and the few listed ones 0 to 6 % for 65,537).  Where the
+    // cell is long and its neighbours lie within the balls they leave nothing out: a cell whose searches with them have
+    // overflowed BALL_FULL times repeats one without them, and if that finds hardly more goes without for one pass, then,
+    // after a few more overflows, for 4, 16 ... (a sheet 1e-3 thick, whose time is that of a few such cells: 105 ms without
+    // balls, 412 ms with them in every search, 120 ms so).
+    int ball_next = A.warp_list ? 1 : BALL_PASS, ball_full = 0, ball_gap = 1;
+    bool over = sizeof(CT) == 8 || A.warp_list;
     for (int pass = 0; pass < A.max_passes && !done; pass++) {
         cc.n_passes++;
         if (rhi2 > cap2) rhi2 = cap2;
         int cnt = -1;
-        const bool balls = BALLS && pass >= (A.warp_list ? 1 : BALL_PASS);
-        if (balls) {
+        bool balls = BALLS && pass >= ball_next && over;
+        int with = -1;  // candidates with the balls, while the search is repeated without them
+        if (BALLS && pass >= ball_next) {
             if (lane == 0)
 #pragma unroll
                 for (int e = 0; e < TP; e++) S.vmk[e] = C.vm[e];
@@ -1353,6 +1365,29 @@ __device__ int do_cell(WarpSmem<CT, TP>& S, const ClipArgs& A, uint32_t self, do
             cc.n_collect++;
             if (cnt > 0) cc.n_collected += cnt;
             if (cnt == -2) return CAP_STACK;
+            if (BALLS && with >= 0) {
+                if (cnt >= 0 && cnt <= K::CAND && 16 * (cnt - with) <= cnt) {
+                    ball_next = pass + 1 + ball_gap;
+                    ball_gap *= 4;
+                    ball_full = BALL_FULL - 4;
+                    break;
+                }
+                balls = true;  // they are worth it
+                with = -1;
+                ball_full = 0;
+                cnt = -1;
+                continue;
+            }
+            if (BALLS && !balls && pass >= ball_next && (cnt == -3 || cnt > K::CAND)) balls = over = true;
+            else if (BALLS && balls) {
+                if (cnt == -3 || cnt > K::CAND) ball_full++;
+                else if (cnt >= 0 && ball_full >= BALL_FULL) {
+                    with = cnt;
+                    balls = false;
+                    cnt = -1;
+                    continue;
+                }
+            }
             if (cnt == -3) {  // aborted: halve the radius step and retry
                 CT r = sqrt(rhi2), rl = sqrt(rlo2);
                 CT rn = rl + (CT)0.5 * (r - rl);
