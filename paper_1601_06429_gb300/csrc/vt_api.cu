@@ -601,8 +601,12 @@ int vt_build_owned(vt_handle* out, const void* pos, int dtype, const void* mass,
     vt_params prm;
     int rc = check_params(p, prm, N);
     if (rc) return rc;
-    // the listed cells go to the lane-group kernel by the library's choice, to the warp kernel otherwise
-    prm.threads_per_cell = p && p->threads_per_cell ? 32 : prm.threads_per_cell;
+    // The owned cells go to the lane groups by the library's choice; to the warp kernel, from a list, if the caller names any
+    // mode and where they are few or few of many, since the groups' first pass goes over all N rows.  By the list and by
+    // groups: 33,000 / 45,000 / 60,000 owned of 300,000 clustered particles 3.24 / 5.32 / 5.65 ms and 4.83 / 5.66 / 6.11 ms,
+    // uniform 2.38 / 3.05 / 3.98 and 2.05 / 2.28 / 2.67 ms; 3000 of 300,000 clustered 0.98 and 2.04 ms; 60,000 of 2,000,000
+    // clustered 6.1 and 10.4 ms, uniform 4.4 both.
+    if ((p && p->threads_per_cell) || n_owned < 40000 || n_owned < N / 32) prm.threads_per_cell = 32;
     Geometry geo;
     rc = make_geometry(box_lo, box_hi, periodic, prm.precision, geo);
     if (rc) return rc;
