@@ -136,6 +136,7 @@ int vt_build(vt_handle *h, const void *pos, int dtype, const void *mass, int64_t
  * the cells of its sub-volume from its own particles plus the boundary particles of a buffer zone around
  * it).  Arguments as vt_build, plus
  *   n_owned  1 <= n_owned <= N: input rows [0, n_owned) are the particles whose cells are computed
+ *            (threads_per_cell 0 takes 4 lanes a cell from n_owned = 40,000 and N / 32 on, N >= 65,536)
  * The handle answers every call of a vt_build handle; the rows of buffer particles have volume 0, density 0,
  * no neighbours, a zero gradient and radius 0, while the neighbour lists of computed cells may name them (input
  * row indices).  A computed cell is the true cell of its particle when every particle within twice its radius

@@ -228,7 +228,7 @@ __device__ __forceinline__ double over_dist(float a, float x, float y, float z) 
     const float s = rsqrtf(dh);
     float p, pr;
     two_prod(a, s, p, pr);
-    if (!(dh > 1e-26f && dh < 1e26f && p > 1e-28f)) {  // outside, the low parts would leave the range of a float
+    if (!(dh > 1e-26f && dh < 1e26f && p > 1e-21f && p < 1e36f)) {  // outside, the low parts would leave the range of a float
         const double X = x, Y = y, Z = z;
         return (double)a / sqrt(fma(Z, Z, fma(Y, Y, X * X)));
     }
@@ -251,7 +251,13 @@ __device__ __forceinline__ double over_dist(float a, float x, float y, float z) 
     float th, tl, uh, ul;
     two_prod(p, hh, th, tl);
     two_sum(pr, th, uh, ul);
-    return f2d(p) + (f2d(uh) + f2d(ul + (tl + fmaf(p, hl, pr * hh))));
+    // (no branch: what lies below the normal floats is below 2^-53 p and taken as zero)
+    auto cvt = [](float v) -> double {
+        const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+        const bool z = m < 0x00800000u;
+        return __hiloint2double(z ? 0 : (int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), z ? 0 : (int)(b << 29));
+    };
+    return cvt(p) + (cvt(uh) + cvt(ul + (tl + fmaf(p, hl, pr * hh))));
 }
 
 // ------------------------------------------------------------------ Green-Gauss gradient
@@ -260,9 +266,9 @@ __device__ __forceinline__ double over_dist(float a, float x, float y, float z) 
 // cell with rho at a facet centroid interpolated linearly between the two sites, exact for a linear field
 // (the tangential parts cancel on a closed Voronoi cell); on a box wall rho is taken as rho_i.  One thread per
 // cell, FP64 sums over FP32 facet records: seven FP64 instructions a facet (FP32 results), and the gathers of records and
-// densities, bound it (one million clustered cells: 625 us; 1465 us with an FP64 root and quotient a facet, 535 us with a
-// quotient to 1e-13 from pairs of floats, which changed the last bit of a result now and then).  FP64 results keep the FP64
-// root and quotient.
+// densities, bound it (one million clustered cells: 490 us; 625 us with branches in the quotient's conversions, 1465 us
+// with an FP64 root and quotient a facet, 535 us with a quotient to 1e-13, which changed the last bit of a result now and
+// then).  FP64 results keep the FP64 root and quotient.
 template <typename T>
 __global__ void k_gradient_gg(const Face* __restrict__ faces, const uint32_t* __restrict__ face_start,
                               const uint16_t* __restrict__ face_count, const CellOut* __restrict__ cell,
